@@ -25,9 +25,9 @@ namespace pm {
 #define PM_DECL_D(D)                                                                                     \
     cudaError_t fused_dispatch_d##D(int, int, const FusedParams &, int, int, size_t, cudaStream_t, int); \
     int fused_blocks_per_sm_d##D(int, int, int, size_t, int);                                            \
-    size_t fused_smem_d##D(int, int, int);                                                               \
-    int fused_groups_per_warp_d##D(int);                                                                 \
-    int fused_max_warps_d##D(int);                                                                       \
+    size_t fused_smem_d##D(int, int, int, int);                                                               \
+    int fused_groups_per_warp_d##D(int, int);                                                                \
+    int fused_max_warps_d##D(int, int);                                                                       \
     cudaError_t grad_run_d##D(int, int, const ScanParams &, const GradParams &, int, int, size_t, cudaStream_t); \
     cudaError_t scan_run_d##D(const ScanParams &, cudaStream_t);                                          \
     int adjoint_blocks_per_sm_d##D(int, int, int, size_t);                                                \
@@ -37,6 +37,13 @@ PM_DECL_D(4)
 PM_DECL_D(8)
 PM_DECL_D(16)
 #undef PM_DECL_D
+#define PM_DECL_FX(D)                                                                                    \
+    cudaError_t fx_basis_d##D(const double *, const double *, int, void *, cudaStream_t);                  \
+    size_t fx_basis_bytes_d##D(int);                                                                     \
+    size_t fx_leaf_bytes_d##D();
+PM_DECL_FX(8)
+PM_DECL_FX(16)
+#undef PM_DECL_FX
 #define PM_DECL_L(D)                                                                                     \
     cudaError_t large_dispatch_d##D(int, int, const FusedParams &, void *, int, size_t, cudaStream_t, int); \
     int large_blocks_per_sm_d##D(int, int, size_t, int);                                                 \
@@ -99,6 +106,7 @@ struct parament_ctx {
     Workspace hraw, full, packed64, packed32, bnorm, partials, tickets, counters, status, check;
     Workspace ctrl_copy, ctrl_conv, uout, bmax, cpacked64, cpacked32, cbnorm;
     Workspace gv, gvdag, gleaf, gblock, gbpin, gpin, gz, gpbuf, gckpt, ggrad, lscratch, gadj;
+    Workspace fxbasis, fxg;  // FP64 digit path: basis digits, packed exponents per leaf
     Workspace tstage, tpsi;  // trajectory: staging of a host output, psi_0 padded (FP64)
     std::vector<double2> tpsi_host;
     // batched plan
@@ -559,12 +567,14 @@ int fused_blocks_per_sm(int Dp, int fp64, int integ, int warps, size_t smem, int
     return memo_occupancy(0, Dp, fp64, integ, warps, smem, cheb,
                           [&] { return fused_blocks_per_sm_uncached(Dp, fp64, integ, warps, smem, cheb); });
 }
-size_t fused_smem(int Dp, int fp64, int nb, int warps) {
+// legacy: the geometry of the FP64 fused kernel on the FP64 pipe (Chebyshev, batched items) where the FP64 Taylor
+// paths run on the digit products
+size_t fused_smem(int Dp, int fp64, int nb, int warps, int legacy = 0) {
     switch (Dp) {
-        case 2: return fused_smem_d2(fp64, nb, warps);
-        case 4: return fused_smem_d4(fp64, nb, warps);
-        case 8: return fused_smem_d8(fp64, nb, warps);
-        case 16: return fused_smem_d16(fp64, nb, warps);
+        case 2: return fused_smem_d2(fp64, nb, warps, legacy);
+        case 4: return fused_smem_d4(fp64, nb, warps, legacy);
+        case 8: return fused_smem_d8(fp64, nb, warps, legacy);
+        case 16: return fused_smem_d16(fp64, nb, warps, legacy);
     }
     return 0;
 }
@@ -682,21 +692,21 @@ size_t large_smem(int Dp, int fp64, int nb, int tc = 0) {
     }
     return 0;
 }
-int fused_max_warps(int Dp, int fp64) {
+int fused_max_warps(int Dp, int fp64, int legacy = 0) {
     switch (Dp) {
-        case 2: return fused_max_warps_d2(fp64);
-        case 4: return fused_max_warps_d4(fp64);
-        case 8: return fused_max_warps_d8(fp64);
-        case 16: return fused_max_warps_d16(fp64);
+        case 2: return fused_max_warps_d2(fp64, legacy);
+        case 4: return fused_max_warps_d4(fp64, legacy);
+        case 8: return fused_max_warps_d8(fp64, legacy);
+        case 16: return fused_max_warps_d16(fp64, legacy);
     }
     return 8;
 }
-int fused_gpw(int Dp, int fp64) {
+int fused_gpw(int Dp, int fp64, int legacy = 0) {
     switch (Dp) {
-        case 2: return fused_groups_per_warp_d2(fp64);
-        case 4: return fused_groups_per_warp_d4(fp64);
-        case 8: return fused_groups_per_warp_d8(fp64);
-        case 16: return fused_groups_per_warp_d16(fp64);
+        case 2: return fused_groups_per_warp_d2(fp64, legacy);
+        case 4: return fused_groups_per_warp_d4(fp64, legacy);
+        case 8: return fused_groups_per_warp_d8(fp64, legacy);
+        case 16: return fused_groups_per_warp_d16(fp64, legacy);
     }
     return 1;
 }
@@ -830,7 +840,7 @@ int parament_destroy(parament_ctx *ctx) {
                             &ctx->gadj,
                             &ctx->bparams, &ctx->binsts, &ctx->btable, &ctx->bitems, &ctx->bfull, &ctx->bpacked,
                             &ctx->bnorms, &ctx->bpartials, &ctx->btickets, &ctx->bcounters, &ctx->bstatus,
-                            &ctx->bqueue, &ctx->bscratch, &ctx->cheb, &ctx->tstage, &ctx->tpsi};
+                            &ctx->bqueue, &ctx->bscratch, &ctx->cheb, &ctx->tstage, &ctx->tpsi, &ctx->fxbasis, &ctx->fxg};
         if (ctx->b_exec) cudaGraphExecDestroy(ctx->b_exec);
         for (Workspace *w : all) ws_free(*w);
     }
@@ -935,6 +945,11 @@ int parament_set_hamiltonians(parament_ctx *ctx, int dim, int n_ctrl, const void
         PM_CUDA(cudaMemcpyAsync((double *)ctx->cbnorm.ptr + sl, (double *)ctx->bnorm.ptr + e, sizeof(double),
                                 cudaMemcpyDeviceToDevice, ctx->stream));
     }
+    if (Dp == 8 || Dp == 16) {
+        if ((st = ws_reserve(ctx, ctx->fxbasis, Dp == 8 ? fx_basis_bytes_d8(kept) : fx_basis_bytes_d16(kept)))) return st;
+        PM_CUDA((Dp == 8 ? fx_basis_d8 : fx_basis_d16)((const double *)ctx->cpacked64.ptr, (const double *)ctx->cbnorm.ptr,
+                                                      kept, ctx->fxbasis.ptr, ctx->stream));
+    }
     ctx->nb_eff = kept;
 
     ctx->dim = dim;
@@ -993,7 +1008,7 @@ namespace {
 // Controls in the compute type, Taylor table and launch geometry of the fused
 // forward kernel (shared by propagate and propagate_grad).
 int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int &grid, int &warps, size_t &smem,
-                  int &leaves_per_block, int tc = 0) {
+                  int &leaves_per_block, int tc = 0, int cheb = 0) {
     const int Dp = ctx->dpad, nb = ctx->nb_eff;
     const void *ctrl = ctx->ctrl;
     const int64_t count = (int64_t)ctx->K * ctx->S;
@@ -1037,31 +1052,31 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
         int st = ws_reserve(ctx, ctx->lscratch, (size_t)grid * 6 * Dp * Dp * csz);
         if (st) return st;
     } else {
-    const int max_warps = fused_max_warps(Dp, fp64);
+    const int max_warps = fused_max_warps(Dp, fp64, cheb);
     warps = (int)ctx->opt_warps;
     if (warps <= 0) {
         warps = max_warps;
-        while (warps > 1 && fused_smem(Dp, fp64, nb, warps) > ctx->smem_optin) --warps;
+        while (warps > 1 && fused_smem(Dp, fp64, nb, warps, cheb) > ctx->smem_optin) --warps;
         if (fp64 && ctx->opt_grid <= 0) {
             // an FP64 slice costs ~64x an FP32 one (GB300's FP64 rate), so a short run is spread
             // over more SMs first: halve the warps per block while the grid that gives every leaf
             // kLeafMinSteps64 slices stays below one block per SM (d = 2, N = 2^14: 8 x 256 ->
             // 128 x 64 threads, 2.2x faster)
             auto blocks_for = [&](int w) {
-                const int64_t per = (int64_t)w * fused_gpw(Dp, fp64) * kLeafMinSteps64;
+                const int64_t per = (int64_t)w * fused_gpw(Dp, fp64, cheb) * kLeafMinSteps64;
                 return (ctx->n_steps + per - 1) / per;
             };
             while (warps > 2 && blocks_for(warps) < ctx->sm_count) warps /= 2;
         }
     }
     if (warps > max_warps) return set_err(ctx, PARAMENT_ERR_INVALID_VALUE, "at most %d warps per block", max_warps);
-    smem = fused_smem(Dp, fp64, nb, warps);
+    smem = fused_smem(Dp, fp64, nb, warps, cheb);
     if (smem > ctx->smem_optin)
         return set_err(ctx, PARAMENT_ERR_UNSUPPORTED, "basis of %d matrices (d=%d) needs %zu B shared memory > %zu",
                        nb, ctx->dim, smem, ctx->smem_optin);
-    const int bps = fused_blocks_per_sm(Dp, fp64, (int)ctx->integ, warps, smem);
+    const int bps = fused_blocks_per_sm(Dp, fp64, (int)ctx->integ, warps, smem, cheb);
     if (bps <= 0) return set_err(ctx, PARAMENT_ERR_CUDA, "occupancy query failed (%d warps, %zu B)", warps, smem);
-    leaves_per_block = warps * fused_gpw(Dp, fp64);
+    leaves_per_block = warps * fused_gpw(Dp, fp64, cheb);
     grid = (int)ctx->opt_grid;
     if (grid <= 0) {
         const int lm = fp64 ? kLeafMinSteps64 : kLeafMinSteps;
@@ -1069,6 +1084,13 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
         grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)bps * ctx->sm_count));
     }
     grid = std::min(grid, ctx->max_grid);
+    if (fp64 && !cheb && Dp >= 8) {
+        const size_t leaf_bytes = Dp == 8 ? fx_leaf_bytes_d8() : fx_leaf_bytes_d16();
+        int st = ws_reserve(ctx, ctx->fxg, (size_t)grid * leaves_per_block * leaf_bytes);
+        if (st) return st;
+        p.fx_basis = ctx->fxbasis.ptr;
+        p.fx_g = ctx->fxg.ptr;
+    }
     }
 
     p.ctrl = ctrl;
@@ -1167,7 +1189,7 @@ int parament_propagate(parament_ctx *ctx, void *U_out, parament_precision prec) 
     int grid = 0, warps = 0, lpb = 0;
     size_t smem = 0;
     const int cheb = ctx->opt_exp_method == 1;
-    int st = forward_setup(ctx, fp64, dst, p, grid, warps, smem, lpb, tc);
+    int st = forward_setup(ctx, fp64, dst, p, grid, warps, smem, lpb, tc, cheb);
     if (st) return st;
     if (cheb) {
         // common spectral half-width over all slices, then degree and coefficients, on the device
@@ -1293,7 +1315,7 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
         const int abps = adjoint_blocks_per_sm(Dp, fp64, (int)ctx->integ, aw, asmem);
         if (abps <= 0) return set_err(ctx, PARAMENT_ERR_CUDA, "adjoint occupancy query failed");
         agrid = abps * ctx->sm_count;
-        TG = (int64_t)agrid * aw * fused_gpw(Dp, fp64);
+        TG = (int64_t)agrid * aw * fused_gpw(Dp, fp64, 1);
     }
     const int64_t maxlen = L > 0 ? (N + L - 1) / L : 0;
     int64_t c_sub = ctx->opt_grad_subchunk > 0 ? ctx->opt_grad_subchunk : std::max<int64_t>(maxlen, 1);
@@ -1624,18 +1646,19 @@ namespace pm {
 
 int fill_classes(double u, int force_m, FusedParams &p) { return build_classes(u, force_m, p); }
 
+// the geometry and kernels that need no workspace (FP64: on the FP64 pipe)
 cudaError_t fused_launch(int Dp, int fp64, int integ, const FusedParams &p, int grid, int warps, size_t smem,
                          cudaStream_t st) {
-    return fused_dispatch(Dp, fp64, integ, p, grid, warps, smem, st);
+    return fused_dispatch(Dp, fp64, integ, p, grid, warps, smem, st, fp64 && Dp >= 8 ? 3 : 0);
 }
 
 int fused_occupancy(int Dp, int fp64, int integ, int warps, size_t smem) {
-    return fused_blocks_per_sm(Dp, fp64, integ, warps, smem);
+    return fused_blocks_per_sm(Dp, fp64, integ, warps, smem, fp64 && Dp >= 8 ? 3 : 0);
 }
 
-size_t fused_smem_size(int Dp, int fp64, int n_basis, int warps) { return fused_smem(Dp, fp64, n_basis, warps); }
+size_t fused_smem_size(int Dp, int fp64, int n_basis, int warps) { return fused_smem(Dp, fp64, n_basis, warps, 1); }
 
-int fused_groups(int Dp, int fp64) { return fused_gpw(Dp, fp64); }
+int fused_groups(int Dp, int fp64) { return fused_gpw(Dp, fp64, 1); }
 
 cudaError_t basis_build(const void *raw, int c128, int d, int Dp, int K, int magnus, int nb, double2 *full,
                         double *p64, float *p32, double *bnorm, double *bmax, cudaStream_t st) {
@@ -1775,10 +1798,10 @@ int batch_run(parament_ctx *ctx, const parament_instance *inst, int n, parament_
             int64_t nb_cap;
             if (Dp[i] <= kMaxSmallDim) {
                 int w = 8;
-                while (w > 1 && fused_smem(Dp[i], fp64, nbs[i], w) > ctx->smem_optin) --w;
+                while (w > 1 && fused_smem(Dp[i], fp64, nbs[i], w, 1) > ctx->smem_optin) --w;
                 warps_of[i] = w;
-                nb_cap = std::max<int64_t>(1, N / ((int64_t)w * fused_gpw(Dp[i], fp64) * leaf_steps));
-                smem = std::max(smem, fused_smem(Dp[i], fp64, nbs[i], w));
+                nb_cap = std::max<int64_t>(1, N / ((int64_t)w * fused_gpw(Dp[i], fp64, 1) * leaf_steps));
+                smem = std::max(smem, fused_smem(Dp[i], fp64, nbs[i], w, 1));
             } else {
                 nb_cap = std::max<int64_t>(1, N / leaf_steps);
                 const int cls = batch_tc_class(Dp[i]);

@@ -81,6 +81,8 @@ struct FusedParams {
     void *traj_out;            // trajectory mode: U(t_n) [n_out][d][d] or psi(t_n) [n_out][d] (U_out's dtype)
     const double2 *traj_psi0;  // trajectory mode: psi_0 padded to D in FP64, or null for U(t_n)
     int64_t traj_every;        // trajectory mode: outputs after slices every, 2 every, ..., and the last
+    const void *fx_basis;      // digit path (pm_fx.cuh): digits of the packed basis
+    void *fx_g;                // digit path: packed exponents of the slices a warp works on, [leaves][16][D][D]
     int n_cls;
     double cls_cap[kMaxClasses];
     int cls_code[kMaxClasses];

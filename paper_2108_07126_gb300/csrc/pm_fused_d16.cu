@@ -1,6 +1,8 @@
 // Instantiations of the fused propagation kernel for padded dimension 16
-// (mode cheb: 0 = Taylor exponential, 1 = Chebyshev exponential, 2 = Taylor trajectory).
-#include "pm_fused.cuh"
+// (mode cheb: 0 = Taylor exponential, 1 = Chebyshev exponential, 2 = Taylor trajectory,
+// 3 = FP64 Taylor on the FP64 pipe for callers without workspace).  FP64 Taylor (0, 2) runs on the
+// exact digit products of pm_fx.cuh; legacy asks for the geometry of the FP64 fused kernel (1, 3, batched items).
+#include "pm_fx.cuh"
 
 namespace pm {
 
@@ -8,11 +10,11 @@ cudaError_t fused_dispatch_d16(int fp64, int integ, const FusedParams &p, int gr
                                cudaStream_t st, int cheb) {
     switch (cheb * 6 + integ * 2 + (fp64 ? 1 : 0)) {
         case 0: return launch_fused<float, 16, kMidpoint>(p, grid, warps, smem, st);
-        case 1: return launch_fused<double, 16, kMidpoint>(p, grid, warps, smem, st);
+        case 1: return fx::launch<16, kMidpoint, false>(p, grid, warps, smem, st);
         case 2: return launch_fused<float, 16, kGL2>(p, grid, warps, smem, st);
-        case 3: return launch_fused<double, 16, kGL2>(p, grid, warps, smem, st);
+        case 3: return fx::launch<16, kGL2, false>(p, grid, warps, smem, st);
         case 4: return launch_fused<float, 16, kSimpson>(p, grid, warps, smem, st);
-        case 5: return launch_fused<double, 16, kSimpson>(p, grid, warps, smem, st);
+        case 5: return fx::launch<16, kSimpson, false>(p, grid, warps, smem, st);
         case 6: return launch_fused<float, 16, kMidpoint, 1>(p, grid, warps, smem, st);
         case 7: return launch_fused<double, 16, kMidpoint, 1>(p, grid, warps, smem, st);
         case 8: return launch_fused<float, 16, kGL2, 1>(p, grid, warps, smem, st);
@@ -20,11 +22,14 @@ cudaError_t fused_dispatch_d16(int fp64, int integ, const FusedParams &p, int gr
         case 10: return launch_fused<float, 16, kSimpson, 1>(p, grid, warps, smem, st);
         case 11: return launch_fused<double, 16, kSimpson, 1>(p, grid, warps, smem, st);
         case 12: return launch_fused<float, 16, kMidpoint, 2>(p, grid, warps, smem, st);
-        case 13: return launch_fused<double, 16, kMidpoint, 2>(p, grid, warps, smem, st);
+        case 13: return fx::launch<16, kMidpoint, true>(p, grid, warps, smem, st);
         case 14: return launch_fused<float, 16, kGL2, 2>(p, grid, warps, smem, st);
-        case 15: return launch_fused<double, 16, kGL2, 2>(p, grid, warps, smem, st);
+        case 15: return fx::launch<16, kGL2, true>(p, grid, warps, smem, st);
         case 16: return launch_fused<float, 16, kSimpson, 2>(p, grid, warps, smem, st);
-        case 17: return launch_fused<double, 16, kSimpson, 2>(p, grid, warps, smem, st);
+        case 17: return fx::launch<16, kSimpson, true>(p, grid, warps, smem, st);
+        case 19: return launch_fused<double, 16, kMidpoint>(p, grid, warps, smem, st);
+        case 21: return launch_fused<double, 16, kGL2>(p, grid, warps, smem, st);
+        case 23: return launch_fused<double, 16, kSimpson>(p, grid, warps, smem, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -32,11 +37,11 @@ cudaError_t fused_dispatch_d16(int fp64, int integ, const FusedParams &p, int gr
 int fused_blocks_per_sm_d16(int fp64, int integ, int warps, size_t smem, int cheb) {
     switch (cheb * 6 + integ * 2 + (fp64 ? 1 : 0)) {
         case 0: return fused_max_blocks_per_sm<float, 16, kMidpoint>(warps, smem);
-        case 1: return fused_max_blocks_per_sm<double, 16, kMidpoint>(warps, smem);
+        case 1: return fx::max_blocks_per_sm<16, kMidpoint, false>(warps, smem);
         case 2: return fused_max_blocks_per_sm<float, 16, kGL2>(warps, smem);
-        case 3: return fused_max_blocks_per_sm<double, 16, kGL2>(warps, smem);
+        case 3: return fx::max_blocks_per_sm<16, kGL2, false>(warps, smem);
         case 4: return fused_max_blocks_per_sm<float, 16, kSimpson>(warps, smem);
-        case 5: return fused_max_blocks_per_sm<double, 16, kSimpson>(warps, smem);
+        case 5: return fx::max_blocks_per_sm<16, kSimpson, false>(warps, smem);
         case 6: return fused_max_blocks_per_sm<float, 16, kMidpoint, 1>(warps, smem);
         case 7: return fused_max_blocks_per_sm<double, 16, kMidpoint, 1>(warps, smem);
         case 8: return fused_max_blocks_per_sm<float, 16, kGL2, 1>(warps, smem);
@@ -44,21 +49,35 @@ int fused_blocks_per_sm_d16(int fp64, int integ, int warps, size_t smem, int che
         case 10: return fused_max_blocks_per_sm<float, 16, kSimpson, 1>(warps, smem);
         case 11: return fused_max_blocks_per_sm<double, 16, kSimpson, 1>(warps, smem);
         case 12: return fused_max_blocks_per_sm<float, 16, kMidpoint, 2>(warps, smem);
-        case 13: return fused_max_blocks_per_sm<double, 16, kMidpoint, 2>(warps, smem);
+        case 13: return fx::max_blocks_per_sm<16, kMidpoint, true>(warps, smem);
         case 14: return fused_max_blocks_per_sm<float, 16, kGL2, 2>(warps, smem);
-        case 15: return fused_max_blocks_per_sm<double, 16, kGL2, 2>(warps, smem);
+        case 15: return fx::max_blocks_per_sm<16, kGL2, true>(warps, smem);
         case 16: return fused_max_blocks_per_sm<float, 16, kSimpson, 2>(warps, smem);
-        case 17: return fused_max_blocks_per_sm<double, 16, kSimpson, 2>(warps, smem);
+        case 17: return fx::max_blocks_per_sm<16, kSimpson, true>(warps, smem);
+        case 19: return fused_max_blocks_per_sm<double, 16, kMidpoint>(warps, smem);
+        case 21: return fused_max_blocks_per_sm<double, 16, kGL2>(warps, smem);
+        case 23: return fused_max_blocks_per_sm<double, 16, kSimpson>(warps, smem);
     }
     return 0;
 }
 
-size_t fused_smem_d16(int fp64, int n_basis, int warps) {
+size_t fused_smem_d16(int fp64, int n_basis, int warps, int legacy) {
+    if (fp64 && !legacy) return fx::smem_bytes<16>(n_basis, warps);
     return fp64 ? fused_smem_bytes<double, 16>(n_basis, warps) : fused_smem_bytes<float, 16>(n_basis, warps);
 }
 
-int fused_groups_per_warp_d16(int fp64) { return fp64 ? Geo<double, 16>::GPW : Geo<float, 16>::GPW; }
+int fused_groups_per_warp_d16(int fp64, int legacy) {
+    return fp64 ? (legacy ? Geo<double, 16>::GPW : 1) : Geo<float, 16>::GPW;
+}
 
-int fused_max_warps_d16(int fp64) { return fp64 ? Geo<double, 16>::MAXW : Geo<float, 16>::MAXW; }
+int fused_max_warps_d16(int fp64, int legacy) {
+    return fp64 ? (legacy ? Geo<double, 16>::MAXW : fx::Cfg<16>::MAXW) : Geo<float, 16>::MAXW;
+}
+
+cudaError_t fx_basis_d16(const double *packed, const double *bnorm, int nb, void *out, cudaStream_t st) {
+    return fx::basis_digits<16>(packed, bnorm, nb, out, st);
+}
+size_t fx_basis_bytes_d16(int nb) { return fx::basis_digit_bytes<16>(nb); }
+size_t fx_leaf_bytes_d16() { return fx::Cfg<16>::LEAF_BYTES; }
 
 }  // namespace pm

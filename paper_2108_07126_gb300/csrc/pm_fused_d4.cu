@@ -53,12 +53,13 @@ int fused_blocks_per_sm_d4(int fp64, int integ, int warps, size_t smem, int cheb
     return 0;
 }
 
-size_t fused_smem_d4(int fp64, int n_basis, int warps) {
+size_t fused_smem_d4(int fp64, int n_basis, int warps, int legacy) {
+    (void)legacy;
     return fp64 ? fused_smem_bytes<double, 4>(n_basis, warps) : fused_smem_bytes<float, 4>(n_basis, warps);
 }
 
-int fused_groups_per_warp_d4(int fp64) { return fp64 ? Geo<double, 4>::GPW : Geo<float, 4>::GPW; }
+int fused_groups_per_warp_d4(int fp64, int) { return fp64 ? Geo<double, 4>::GPW : Geo<float, 4>::GPW; }
 
-int fused_max_warps_d4(int fp64) { return fp64 ? Geo<double, 4>::MAXW : Geo<float, 4>::MAXW; }
+int fused_max_warps_d4(int fp64, int) { return fp64 ? Geo<double, 4>::MAXW : Geo<float, 4>::MAXW; }
 
 }  // namespace pm
