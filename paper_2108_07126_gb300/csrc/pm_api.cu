@@ -1135,9 +1135,9 @@ void record_launch(parament_ctx *ctx, int nb, int grid, int warps, int leaves_pe
     ctx->last.kernel_ms = -1.0;
 }
 
-// V^dagger, padded with zeros to Dp x Dp, in FP64
+// V^dagger, padded with zeros to Dp x Dp, in FP64; clears the norm bound of vnorm_kernel
 template <typename InT>
-__global__ void vdag_kernel(const InT *V, int d, int Dp, double2 *out) {
+__global__ void vdag_kernel(const InT *V, int d, int Dp, double2 *out, double *z) {
     for (int t = threadIdx.x; t < Dp * Dp; t += blockDim.x) {
         const int i = t / Dp, j = t % Dp;
         double2 v = make_double2(0.0, 0.0);
@@ -1147,6 +1147,29 @@ __global__ void vdag_kernel(const InT *V, int d, int Dp, double2 *out) {
         }
         out[t] = v;
     }
+    if (threadIdx.x == 0) z[3] = 0.0;
+}
+
+// z[3] = max_i sum_j |(V^dagger V)_ij| >= ||V||_2^2 (one for a unitary V): bounds the matrices of the adjoint sweep,
+// whose fixed-point products need entries below two.  Block i: row i.
+__global__ void __launch_bounds__(128) vnorm_kernel(const double2 *vdag, int d, int Dp, double *z) {
+    const int i = blockIdx.x;
+    double s = 0.0;
+    for (int j = threadIdx.x; j < d; j += blockDim.x) {
+        double2 acc = make_double2(0.0, 0.0);
+        for (int k = 0; k < d; ++k) {  // vdag[i][k] * conj(vdag[j][k])
+            const double2 a = vdag[(size_t)i * Dp + k], b = vdag[(size_t)j * Dp + k];
+            acc.x = fma(a.x, b.x, fma(a.y, b.y, acc.x));
+            acc.y = fma(a.y, b.x, fma(-a.x, b.y, acc.y));
+        }
+        s += sqrt(acc.x * acc.x + acc.y * acc.y);
+    }
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    __shared__ double part[4];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        atomicMax((unsigned long long *)(z + 3), dbits(part[0] + part[1] + part[2] + part[3]));
 }
 
 // psi_0 padded with zeros to Dp entries, in FP64
@@ -1263,11 +1286,18 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
         Vd = ctx->gv.ptr;
     }
     if ((st = ws_reserve(ctx, ctx->gvdag, DD * sizeof(double2)))) return st;
+    if ((st = ws_reserve(ctx, ctx->gz, 4 * sizeof(double)))) return st;
     if (ctx->dtype == PARAMENT_C128)
-        vdag_kernel<double2><<<1, 256, 0, ctx->stream>>>((const double2 *)Vd, d, Dp, (double2 *)ctx->gvdag.ptr);
+        vdag_kernel<double2><<<1, 256, 0, ctx->stream>>>((const double2 *)Vd, d, Dp, (double2 *)ctx->gvdag.ptr,
+                                                        (double *)ctx->gz.ptr);
     else
-        vdag_kernel<float2><<<1, 256, 0, ctx->stream>>>((const float2 *)Vd, d, Dp, (double2 *)ctx->gvdag.ptr);
+        vdag_kernel<float2><<<1, 256, 0, ctx->stream>>>((const float2 *)Vd, d, Dp, (double2 *)ctx->gvdag.ptr,
+                                                       (double *)ctx->gz.ptr);
     PM_CUDA(cudaGetLastError());
+    if (Dp > kMaxSmallDim) {
+        vnorm_kernel<<<d, 128, 0, ctx->stream>>>((const double2 *)ctx->gvdag.ptr, d, Dp, (double *)ctx->gz.ptr);
+        PM_CUDA(cudaGetLastError());
+    }
 
     // forward pass keeping every leaf and block product
     const bool host_u = U_out && !is_device_ptr(U_out);
@@ -1280,7 +1310,6 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     const int64_t L = (int64_t)grid * lpb;
     const bool large = Dp > kMaxSmallDim;  // one leaf per thread block, block-level adjoint
     if ((st = ws_reserve(ctx, ctx->gleaf, (size_t)L * DD * sizeof(double2)))) return st;
-    if ((st = ws_reserve(ctx, ctx->gz, 4 * sizeof(double)))) return st;
     p.leaf_out = (double2 *)ctx->gleaf.ptr;
     if (large) {
         // prefix scan over L + 1 elements (the last prefix is U(T)) and suffix scan, ping-pong each

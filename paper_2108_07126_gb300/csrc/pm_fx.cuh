@@ -7,12 +7,14 @@
 // are kept as 64-bit fixed-point numbers x = q 2^-56 (absolute rounding 2^-57, less than the rounding of a
 // double near 1/4), and a product needs no scaling:
 //   * q is split into seven balanced base-256 digits (the top one has 10 bits, |x| < 2), each an exact f16;
-//   * digit products are summed by mma.sync m16n8k16 (f16 in, f32 accumulate).  The sums are integers
-//     below 2^22 (worst case over 32 real terms, 28 digit pairs i + j <= 6), so every f32 accumulation is
+//   * digit products are summed by mma.sync m16n8k16 (f16 in, f32 accumulate), one accumulator per diagonal
+//     i + j = t.  The sums are integers below 2^22 (worst case over 32 real terms), so every f32 accumulation is
 //     exact; with the accumulator started at 1.5 2^23 the integer can be read from the bits of the float;
-//   * the seven diagonal sums are added in 64-bit integers; dropped digit pairs are below 2^-57.
+//   * the diagonal sums t = 0 .. 7 (34 digit pairs) are added in 64-bit integers.  The dropped ones (t >= 8) are below
+//     2^-62; without t = 7 (28 pairs) a 16 x 16 product was off by 2^-56, a 128 x 128 one by 2^-54, more than on the FP64
+//     pipe.
 // The FP64 pipe of GB300 runs about two multiply-adds per clock and SM, mma.sync 1024: one 16 x 16 complex
-// product takes 9.7 k SM cycles on the FP64 pipe and 224 MMAs (450 cycles) here.
+// product takes 9.7 k SM cycles on the FP64 pipe and 272 MMAs (550 cycles) here.
 //
 // Register layout (one warp per matrix).  Lane 4 g + t holds, for D = 16, the pairs of entries
 // (row g + 8 r, columns 8 h + 2 t, + 1), pair index 2 h + r, and for D = 8 the pair (row g, columns 2 t, + 1):
@@ -36,6 +38,7 @@ typedef unsigned long long u64;
 
 constexpr int F = 56;     // fraction bits
 constexpr int ND = 7;     // digits
+constexpr int NA = 8;     // diagonals i + j of digit pairs that are summed (0 .. 7)
 constexpr float kBias = 12582912.f;             // 1.5 * 2^23: floats in [2^23, 2^24) have integer spacing
 constexpr u64 kSplitBias = 0x0200808080808080ull;  // makes every digit field non-negative
 
@@ -48,14 +51,14 @@ __device__ __forceinline__ i64 from_double(double v, int s) {  // round(v 2^(F -
     else q = sh > -60 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0ull;
     return b < 0 ? -(i64)q : (i64)q;
 }
-// q 2^-56 rounded to a double, in integer arithmetic (the conversion instruction runs on the FP64 pipe, 16 cycles a warp)
-__device__ __forceinline__ double to_double(i64 q) {
+// q 2^-FR rounded to a double, in integer arithmetic (the conversion instruction runs on the FP64 pipe, 16 cycles a warp)
+template <int FR = F> __device__ __forceinline__ double to_double(i64 q) {
     const u64 a = q < 0 ? (u64)-q : (u64)q;
     if (a == 0) return 0.0;
     const int lz = __clzll((long long)a);
     const u64 m = a << lz;
     const u64 mant = (m >> 11) + ((m >> 10) & 1);  // 53 bits, the leading one adds to the exponent
-    const u64 bits = ((u64)(1023 + 63 - F - 1 - lz) << 52) + mant;
+    const u64 bits = ((u64)(1023 + 63 - FR - 1 - lz) << 52) + mant;
     return __longlong_as_double((long long)(bits | ((u64)q & 0x8000000000000000ull)));
 }
 
@@ -140,7 +143,7 @@ __device__ __forceinline__ uint32_t transpose8(uint32_t w) {
 // The right operand of a product, as the digits of its transpose, in shared memory that is private to the
 // lane: word (digit, part, pair) at ((digit * 2 + part) * NP + pair) * 32 + lane.
 constexpr int kPlain = 0, kAntiHerm = 1, kHerm = 2, kTrans = 3;
-template <int D> constexpr int rhs_words() { return ND * 2 * L<D>::NP * 32; }
+template <int D> __host__ __device__ constexpr int rhs_words() { return ND * 2 * L<D>::NP * 32; }
 
 // digits of M (own layout) -> right operand: kPlain: M^T as B; kAntiHerm: M^T = -conj(M); kHerm: M^T = conj(M);
 // kTrans: transposed through movmatrix
@@ -183,27 +186,46 @@ __device__ __forceinline__ void mma_first(float (&c)[4], uint32_t a0, uint32_t a
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(s));
 }
 
-__device__ __forceinline__ void acc_init(float (&acc)[ND][4]) {
+__host__ __device__ constexpr float acc_start(int t) { return t < 6 ? kBias : 0.f; }
+// last digit j paired with digit i
+__host__ __device__ constexpr int last_digit(int i) { return NA - 1 - i < ND - 1 ? NA - 1 - i : ND - 1; }
+// whether the pair (i, j) is the first on its diagonal in the loops over i, then j
+__host__ __device__ constexpr bool first_pair(int i, int j) { return i == 0 || (j == ND - 1 && i + j < NA); }
+
+__device__ __forceinline__ void acc_init(float (&acc)[NA][4]) {
 #pragma unroll
-    for (int t = 0; t < ND; ++t)
+    for (int t = 0; t < NA; ++t)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[t][u] = t < ND - 1 ? kBias : 0.f;
+        for (int u = 0; u < 4; ++u) acc[t][u] = acc_start(t);
 }
 
-// sum_t v_t 2^(40 - 8 t) of the diagonal sums v_t = i + j = t; v_0 .. v_5 biased, v_6 plain (rounded to 2^-56)
-__device__ __forceinline__ i64 collect(const float (&acc)[ND][4], int u) {
+// sum_t v_t 2^(40 - 8 t) of the diagonal sums v_t; v_0 .. v_5 biased, v_6 and v_7 plain (rounded to 2^-56)
+__device__ __forceinline__ i64 collect(const float (&acc)[NA][4], int u) {
     constexpr uint32_t B = 0x4B400000u, C = 257u * B;  // 256 B + B mod 2^32
-    const uint32_t w5 = __float_as_uint(fmaf(acc[6][u], 0.00390625f, acc[5][u]));  // v_5 + round(v_6 / 256), biased
+    // v_5 + round((v_6 + v_7 / 256) / 256), biased
+    const uint32_t w5 = __float_as_uint(fmaf(fmaf(acc[7][u], 0.00390625f, acc[6][u]), 0.00390625f, acc[5][u]));
     const int32_t lo = (int32_t)(__float_as_uint(acc[4][u]) * 256u + w5 - C);
     const int32_t mid = (int32_t)(__float_as_uint(acc[2][u]) * 256u + __float_as_uint(acc[3][u]) - C);
     const uint32_t hi = __float_as_uint(acc[0][u]) * 256u + __float_as_uint(acc[1][u]) - C;
     return (i64)mid * 65536 + (i64)lo + (i64)((u64)hi << 32);
 }
 
+// the same sum rounded to 2^-60: for outputs that are collected panel by panel
+constexpr int FC = 60;
+__device__ __forceinline__ i64 collect_fine(const float (&acc)[NA][4], int u) {
+    constexpr uint32_t B = 0x4B400000u, C = 257u * B;
+    const uint32_t b6 = __float_as_uint(fmaf(acc[7][u], 0.00390625f, acc[6][u]) + kBias);
+    const int32_t l = (int32_t)(__float_as_uint(acc[5][u]) * 256u + b6 - C);
+    const int32_t m = (int32_t)(__float_as_uint(acc[3][u]) * 256u + __float_as_uint(acc[4][u]) - C);
+    const int32_t h = (int32_t)(__float_as_uint(acc[1][u]) * 256u + __float_as_uint(acc[2][u]) - C);
+    const uint32_t t = __float_as_uint(acc[0][u]) - B;
+    return (i64)((l + 8) >> 4) + (i64)m * 4096 + (i64)h * (1 << 28) + (i64)((u64)t << 44);
+}
+
 // one quarter of a 16 x 16 product: n-tile nt (columns 8 nt ..), part 0 = Re, 1 = Im -> o[2 r + c]
 __device__ __forceinline__ void mul16_quarter(const Digits<16> &a, const uint32_t *rhs, int lane, int nt, int part,
                                               i64 (&o)[4]) {
-    float acc[ND][4];
+    float acc[NA][4];
     // Re: Ar Br + Ai (-Bi); Im: Ar Bi + Ai Br
     const uint32_t f2 = part ? 0u : 0x80008000u;
     {
@@ -216,8 +238,8 @@ __device__ __forceinline__ void mul16_quarter(const Digits<16> &a, const uint32_
 #pragma unroll
         for (int i = 0; i < ND; ++i)
 #pragma unroll
-            for (int j = 0; j < ND - i; ++j) {
-                if (i == 0) mma_first(acc[j], a.re[0][0], a.re[0][1], a.re[0][2], a.re[0][3], b[j][0], b[j][1], j < ND - 1 ? kBias : 0.f);
+            for (int j = 0; j <= last_digit(i); ++j) {
+                if (first_pair(i, j)) mma_first(acc[i + j], a.re[i][0], a.re[i][1], a.re[i][2], a.re[i][3], b[j][0], b[j][1], acc_start(i + j));
                 else mma(acc[i + j], a.re[i][0], a.re[i][1], a.re[i][2], a.re[i][3], b[j][0], b[j][1]);
             }
     }
@@ -231,7 +253,7 @@ __device__ __forceinline__ void mul16_quarter(const Digits<16> &a, const uint32_
 #pragma unroll
         for (int i = 0; i < ND; ++i)
 #pragma unroll
-            for (int j = 0; j < ND - i; ++j)
+            for (int j = 0; j <= last_digit(i); ++j)
                 mma(acc[i + j], a.im[i][0], a.im[i][1], a.im[i][2], a.im[i][3], b[j][0], b[j][1]);
     }
 #pragma unroll
@@ -251,7 +273,7 @@ __device__ __forceinline__ void mul(const Digits<16> &a, const uint32_t *rhs, in
     }
 }
 __device__ __forceinline__ void mul(const Digits<8> &a, const uint32_t *rhs, int lane, Tile<8> &o) {
-    float acc[ND][4];
+    float acc[NA][4];
     uint32_t b[ND][2];
 #pragma unroll
     for (int j = 0; j < ND; ++j) {
@@ -262,8 +284,8 @@ __device__ __forceinline__ void mul(const Digits<8> &a, const uint32_t *rhs, int
     for (int i = 0; i < ND; ++i) {
         const uint32_t n = neg2(a.im[i][0]);
 #pragma unroll
-        for (int j = 0; j < ND - i; ++j) {
-            if (i == 0) mma_first(acc[j], a.re[0][0], a.im[0][0], n, a.re[0][0], b[j][0], b[j][1], j < ND - 1 ? kBias : 0.f);
+        for (int j = 0; j <= last_digit(i); ++j) {
+            if (first_pair(i, j)) mma_first(acc[i + j], a.re[i][0], a.im[i][0], n, a.re[i][0], b[j][0], b[j][1], acc_start(i + j));
             else mma(acc[i + j], a.re[i][0], a.im[i][0], n, a.re[i][0], b[j][0], b[j][1]);
         }
     }
@@ -361,12 +383,10 @@ __global__ void __launch_bounds__(32) basis_digits_kernel(const double *packed, 
 // for 16 basis matrices at D = 16, here 56 MMAs (112 cycles).  Sums over more than 32 matrices are collected
 // every 32 (the exactness bound).
 template <int D>
-__device__ __forceinline__ void assemble(const FusedParams &p, const double *gam, const int *cls, const double *bnorm,
-                                         int lane, i64 *g) {
+__device__ __forceinline__ void assemble_tile(const uint2 *bd, int nb, const double *gam, int s0, int s1,
+                                              const double *bnorm, int lane, i64 *g) {
     constexpr int DD = D * D, NT = DD / 8;
-    const int nb = p.n_basis, gr = lane >> 2, t4 = lane & 3;
-    const int s0 = cls_s(p.cls_code[cls[gr]]) + p.extra_squarings, s1 = cls_s(p.cls_code[cls[gr + 8]]) + p.extra_squarings;
-    const uint2 *bd = (const uint2 *)p.fx_basis;
+    const int gr = lane >> 2, t4 = lane & 3;  // the lane's rows: slices gr and gr + 8, squarings s0 and s1
     for (int k0 = 0; k0 < 16 * ksteps(nb); k0 += 32) {
         uint32_t a[2][4][ND];
 #pragma unroll
@@ -391,7 +411,7 @@ __device__ __forceinline__ void assemble(const FusedParams &p, const double *gam
         for (int j = 0; j < ND; ++j) b[j] = __ldg(bk + j * 32);
 #pragma unroll 1
         for (int nt = 0; nt < NT; ++nt) {
-            float acc[ND][4];
+            float acc[NA][4];
             uint2 c[ND];
             const int last = (nt + 1 < NT ? nt + 1 : nt) * ND * 32;
 #pragma unroll
@@ -399,8 +419,8 @@ __device__ __forceinline__ void assemble(const FusedParams &p, const double *gam
 #pragma unroll
             for (int i = 0; i < ND; ++i)
 #pragma unroll
-                for (int j = 0; j < ND - i; ++j) {
-                    if (i == 0) mma_first(acc[j], a[0][0][0], a[0][1][0], a[0][2][0], a[0][3][0], b[j].x, b[j].y, j < ND - 1 ? kBias : 0.f);
+                for (int j = 0; j <= last_digit(i); ++j) {
+                    if (first_pair(i, j)) mma_first(acc[i + j], a[0][0][i], a[0][1][i], a[0][2][i], a[0][3][i], b[j].x, b[j].y, acc_start(i + j));
                     else mma(acc[i + j], a[0][0][i], a[0][1][i], a[0][2][i], a[0][3][i], b[j].x, b[j].y);
                 }
 #pragma unroll
@@ -411,7 +431,7 @@ __device__ __forceinline__ void assemble(const FusedParams &p, const double *gam
 #pragma unroll
                 for (int i = 0; i < ND; ++i)
 #pragma unroll
-                    for (int j = 0; j < ND - i; ++j)
+                    for (int j = 0; j <= last_digit(i); ++j)
                         mma(acc[i + j], a[1][0][i], a[1][1][i], a[1][2][i], a[1][3][i], c[j].x, c[j].y);
             }
             i64 o[4];
@@ -491,7 +511,8 @@ __global__ void __launch_bounds__(Cfg<D>::MAXW * 32, 1) fx_kernel(const FusedPar
         }
         __syncwarp();
         const int nr = min(kGT, len - t0);
-        assemble<D>(p, gam, cls, bnorm, lane, gbuf);
+        assemble_tile<D>((const uint2 *)p.fx_basis, nb, gam, cls_s(p.cls_code[cls[lane >> 2]]) + p.extra_squarings,
+                         cls_s(p.cls_code[cls[(lane >> 2) + 8]]) + p.extra_squarings, bnorm, lane, gbuf);
         __syncwarp();
         longlong2 gq[EPL / 2];  // the next slice's packed exponent
         auto fetch = [&](int rr) {

@@ -38,10 +38,10 @@ struct GradParams {
     short slot_of[kMaxBasis];
     const void *packed;      // Real [n_basis][D][D] packed basis (kept matrices)
     const double *bnorm1;    // [n_basis]
-    const double2 *pin;      // [L][D][D] exclusive prefix of each leaf
+    const double2 *pin;      // [L][D][D] exclusive prefix of each leaf (D = 8, 16: [L + 1], the last is U(T))
     const double2 *sout;     // [L][D][D] exclusive suffix of each leaf
     const double2 *vdag;     // [D][D] V^dagger (padded with zeros)
-    const double *z;         // z = Tr(V^dagger U): z[0] + i z[1]
+    const double *z;         // z = Tr(V^dagger U): z[0] + i z[1]; z[3]: bound on ||V||_2^2
     void *grad;              // Real [K][S], zeroed before the launch (Simpson end points add up)
     void *pbuf;              // Real complex [groups][c_sub][D][D]: prefixes of one sub-chunk
     void *ckpt;              // Real complex [groups][n_ckpt][D][D]: sub-chunk checkpoints
@@ -57,6 +57,8 @@ struct GradParams {
     int dcls_code[kMaxClasses];
     double coef_d[kMaxDegree + 1];
     float coef_f[kMaxDegree + 1];
+    const void *fx_basis, *fx_trace;  // digit path (pm_fx_grad.cuh): digits of the basis for the exponents and the traces
+    void *fx_g;                       // digit path: workspace per leaf
 };
 
 struct ScanParams {

@@ -14,6 +14,7 @@
 #include <type_traits>
 
 #include "pm_fused.cuh"
+#include "pm_fxl.cuh"
 #include "pm_tc_small.cuh"
 #include "pm_umma.cuh"
 
@@ -53,11 +54,16 @@ template <typename Real, int D> struct LGeo {
 // shared-memory body of pm_tc_small.cuh (D = 32, 64)
 template <int TCM> __host__ __device__ constexpr int tcm_format() { return (TCM == 3 || TCM == 5) ? umma::kBF16x3 : umma::kTF32x3; }
 
+// FP64 levels of the arrival tree on the digit products in the FP32 kernels too: where their shared memory holds
+// the digit panels anyway (D = 32, 64; at D = 128 the panels would cost the FP32 kernel its second block per SM)
+template <int D> __host__ __device__ constexpr bool tree_on_digits() { return D <= 64; }
+
 template <typename Real, int D, int TCM = 0>
 __host__ __device__ inline size_t large_panel_bytes() {
     // the FP64 top tree and the tensor-core products run through the same panels
     size_t b = LGeo<Real, D>::PANEL_BYTES;
     if (LGeo<double, D>::PANEL_BYTES > b) b = LGeo<double, D>::PANEL_BYTES;
+    if ((std::is_same<Real, double>::value || tree_on_digits<D>()) && fxl::mm_bytes<D>() > b) b = fxl::mm_bytes<D>();
     if (TCM >= 2 && umma::kSmemBytes > b) b = umma::kSmemBytes;
     return b;
 }
@@ -82,7 +88,7 @@ __host__ __device__ inline size_t large_smem_bytes(int n_basis) {
     if constexpr (TCM >= 4) {
         // the tensor-core body, and the FP64 / FP32 panels of the arrival tree that may follow it
         size_t b = tcs::smem_bytes<D, tcm_format<TCM>()>(n_basis);
-        if (LGeo<double, D>::PANEL_BYTES > b) b = LGeo<double, D>::PANEL_BYTES;
+        if (fxl::mm_bytes<D>() > b) b = fxl::mm_bytes<D>();
         return (b + 15) & ~(size_t)15;
     }
     size_t b = large_front_bytes<Real, D, TCM>() + (size_t)(n_basis + 1) * sizeof(Real) + 64;
@@ -220,7 +226,8 @@ __device__ __forceinline__ void smem_mm(const float2 *__restrict__ A, const floa
 // in four 128 x 128 output blocks over K = 256
 template <typename Real, int D, int TCM>
 __device__ __forceinline__ void large_mm(const typename Cx<Real>::T *A, const typename Cx<Real>::T *B,
-                                         typename Cx<Real>::T *Cout, unsigned char *panels, umma::Ctx *uc) {
+                                         typename Cx<Real>::T *Cout, unsigned char *panels, umma::Ctx *uc,
+                                         bool cheb = false) {
     if constexpr ((TCM == 2 || TCM == 3) && std::is_same<Real, float>::value) {
         constexpr int F = TCM == 3 ? umma::kBF16x3 : umma::kTF32x3;
         if constexpr (D == 128) {
@@ -235,6 +242,10 @@ __device__ __forceinline__ void large_mm(const typename Cx<Real>::T *A, const ty
         }
     } else if constexpr (large_resident<Real, D, TCM>()) {
         smem_mm<D>(A, B, Cout);
+    } else if constexpr (std::is_same<Real, double>::value) {
+        // digit products; the Clenshaw recurrence of the Chebyshev series leaves their range (|entry| < 2)
+        if (cheb) cta_mm<Real, D>(A, B, Cout, panels);
+        else fxl::cta_mm<D>(A, B, Cout, panels);
     } else {
         cta_mm<Real, D>(A, B, Cout, panels);
     }
@@ -358,7 +369,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             }
             __syncthreads();
             for (int k = mch - 1; k >= 0; --k) {
-                large_mm<Real, D, TCM>(SX, d1, nw, panels, uc);
+                large_mm<Real, D, TCM>(SX, d1, nw, panels, uc, true);
                 const C a_k = ak[k];
                 for (int e = tid; e < DD; e += kLargeThreads) {
                     const C x = nw[e], y = d2[e];
@@ -378,7 +389,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
                 }
             }
             // leaf product R <- U_j R into P1 (U_j is in one of SX2, SX3, P0), which becomes R
-            large_mm<Real, D, TCM>(nw, SR, P1, panels, uc);
+            large_mm<Real, D, TCM>(nw, SR, P1, panels, uc, true);
             {
                 C *old = SR;
                 SR = P1;
@@ -607,7 +618,8 @@ __device__ void large_arrival_tree(const FusedParams &p, void *ws_bytes, int blk
                     R2[e] = __ldcg(gR + e);
                 }
                 __syncthreads();
-                cta_mm<double, D>(R2, L2, gL, smem);
+                if constexpr (std::is_same<Real, double>::value || tree_on_digits<D>()) fxl::cta_mm<D>(R2, L2, gL, smem);
+                else cta_mm<double, D>(R2, L2, gL, smem);
             } else {
                 float2 *Lf = (float2 *)ws_bytes, *Rf = Lf + DD, *Cf = Rf + DD;
                 for (int e = tid; e < DD; e += kLargeThreads) {
@@ -711,6 +723,41 @@ __global__ void __launch_bounds__(256) tree_level_kernel(const double2 *__restri
     }
 }
 
+// The same level with FP64 products on the digit products: block (tile, pair) computes one 32 x 32 tile.
+// D = 128, one product: 16 blocks of 14 k cycles against 16 blocks of 308 k on the FP64 pipe.
+template <int D>
+__global__ void __launch_bounds__(256) tree_level_fx_kernel(const double2 *__restrict__ in, int n_in,
+                                                            double2 *__restrict__ out, const FusedParams p) {
+    constexpr int T = 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int ti = blockIdx.x / (D / T), tj = blockIdx.x % (D / T), pair = blockIdx.y;
+    const size_t DD = (size_t)D * D;
+    const double2 *L = in + (size_t)(2 * pair) * DD, *R = L + DD;  // earlier, later
+    double2 *O = out + (size_t)pair * DD + (size_t)(ti * T) * D + tj * T;
+    if (2 * pair + 1 < n_in) {
+        fxl::block_mm<T>(R + (size_t)(ti * T) * D, D, L + tj * T, D, O, D, D, smem);
+    } else {
+        for (int e = threadIdx.x; e < T * T; e += blockDim.x)
+            O[(size_t)(e / T) * D + e % T] = L[(size_t)(ti * T + e / T) * D + tj * T + e % T];
+        __syncthreads();
+    }
+    if (gridDim.y == 1 && n_in <= 2) {  // last level: the propagator itself
+        const int d = p.d_out;
+        for (int e = threadIdx.x; e < T * T; e += blockDim.x) {
+            const int i = ti * T + e / T, j = tj * T + e % T;
+            if (i < d && j < d) {
+                const double2 v = O[(size_t)(e / T) * D + e % T];
+                if (p.out_c128) ((double2 *)p.U_out)[i * d + j] = v;
+                else ((float2 *)p.U_out)[i * d + j] = make_float2((float)v.x, (float)v.y);
+            }
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            for (int i = 0; i < 4; ++i) p.counters[4 + i] = atomicExch(&p.counters[i], 0ull);
+            p.status[1] = atomicExch(&p.status[0], 0u);
+        }
+    }
+}
+
 // Exclusive prefixes of the leaf products for the trajectory pass, by a Hillis-Steele scan in
 // FP64: x_0 = I, x_b = leaf_{b-1}; at each level out_i = in_i in_{i-off} for i >= off (the later
 // factor on the left), off = 1, 2, 4, ...; the result is prefix_b = leaf_{b-1} ... leaf_0.
@@ -724,49 +771,28 @@ __global__ void __launch_bounds__(256) prefix_init_kernel(const double2 *__restr
     }
 }
 
-// one level: block (tile, i) computes one 32 x 32 tile of out_i
+// one level: block (tile, i) computes one 32 x 32 tile of out_i on the digit products (pm_fxl.cuh)
 template <int D>
 __global__ void __launch_bounds__(256) prefix_level_kernel(const double2 *__restrict__ in, int n, int off,
                                                            double2 *__restrict__ out) {
-    constexpr int T = 32, KP = 16;
-    __shared__ double2 As[T][KP + 1], Bs[KP][T + 1];
-    const int tiles = D / T;
-    const int ti = blockIdx.x / tiles, tj = blockIdx.x % tiles, i = blockIdx.y;
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+    constexpr int T = 32;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int ti = blockIdx.x / (D / T), tj = blockIdx.x % (D / T), i = blockIdx.y;
     const size_t DD = (size_t)D * D;
     const double2 *Lt = in + (size_t)i * DD;  // later factor (left)
-    double2 *O = out + (size_t)i * DD;
+    double2 *O = out + (size_t)i * DD + (size_t)(ti * T) * D + tj * T;
     if (i < off) {
-        for (int e = threadIdx.x; e < T * T; e += blockDim.x) {
-            const size_t at = (size_t)(ti * T + e / T) * D + tj * T + e % T;
-            O[at] = Lt[at];
-        }
+        for (int e = threadIdx.x; e < T * T; e += blockDim.x)
+            O[(size_t)(e / T) * D + e % T] = Lt[(size_t)(ti * T + e / T) * D + tj * T + e % T];
         return;
     }
     const double2 *Rt = in + (size_t)(i - off) * DD;  // earlier factor (right)
-    double2 acc[2][2] = {{make_double2(0.0, 0.0), make_double2(0.0, 0.0)}, {make_double2(0.0, 0.0), make_double2(0.0, 0.0)}};
-    for (int k0 = 0; k0 < D; k0 += KP) {
-        for (int e = threadIdx.x; e < T * KP; e += blockDim.x) {
-            const int r = e / KP, k = e % KP;
-            As[r][k] = Lt[(size_t)(ti * T + r) * D + k0 + k];
-            const int kb = e / T, cb = e % T;
-            Bs[kb][cb] = Rt[(size_t)(k0 + kb) * D + tj * T + cb];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < KP; ++k) {
-            const double2 a0 = As[ty][k], a1 = As[ty + 16][k], b0 = Bs[k][tx], b1 = Bs[k][tx + 16];
-            cfma(acc[0][0], a0, b0);
-            cfma(acc[0][1], a0, b1);
-            cfma(acc[1][0], a1, b0);
-            cfma(acc[1][1], a1, b1);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) O[(size_t)(ti * T + ty + 16 * r) * D + tj * T + tx + 16 * c] = acc[r][c];
+    fxl::block_mm<T>(Lt + (size_t)(ti * T) * D, D, Rt + tj * T, D, O, D, D, smem);
+}
+
+// the kernels above use more than the default limit of dynamic shared memory
+template <typename K> cudaError_t allow_block_mm_smem(K k) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fxl::G<32>::BYTES);
 }
 
 // exclusive prefixes of n leaf products into x (one of the two buffers a, b; returned)
@@ -774,9 +800,10 @@ template <int D>
 cudaError_t leaf_prefixes(const double2 *leaf, int n, double2 *a, double2 *b, double2 **x, cudaStream_t st) {
     prefix_init_kernel<D><<<1024, 256, 0, st>>>(leaf, n, a);
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = allow_block_mm_smem(prefix_level_kernel<D>);
     double2 *cur = a, *nxt = b;
     for (int off = 1; off < n && e == cudaSuccess; off <<= 1) {
-        prefix_level_kernel<D><<<dim3((D / 32) * (D / 32), n), 256, 0, st>>>(cur, n, off, nxt);
+        prefix_level_kernel<D><<<dim3((D / 32) * (D / 32), n), 256, fxl::G<32>::BYTES, st>>>(cur, n, off, nxt);
         e = cudaGetLastError();
         double2 *t = cur;
         cur = nxt;
@@ -796,13 +823,14 @@ cudaError_t launch_large(const FusedParams &p, void *scratch, int grid, size_t s
     k<<<grid, kLargeThreads, smem, st>>>(p, scratch);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (p.traj_out) return cudaSuccess;  // trajectory pass: no tree
+    if ((e = allow_block_mm_smem(tree_level_fx_kernel<D>)) != cudaSuccess) return e;
     double2 *bufs[2] = {p.partials, (double2 *)scratch};
     int cur = 0, n = grid;
     do {
         const int n_out = (n + 1) / 2;
         const dim3 g((D / 32) * (D / 32), n_out);
         if (std::is_same<Real, double>::value || n <= 8)
-            tree_level_kernel<double, D><<<g, 256, 0, st>>>(bufs[cur], n, bufs[cur ^ 1], p);
+            tree_level_fx_kernel<D><<<g, 256, fxl::G<32>::BYTES, st>>>(bufs[cur], n, bufs[cur ^ 1], p);
         else
             tree_level_kernel<float, D><<<g, 256, 0, st>>>(bufs[cur], n, bufs[cur ^ 1], p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
