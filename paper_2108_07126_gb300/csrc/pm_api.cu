@@ -40,6 +40,9 @@ PM_DECL_D(16)
 #define PM_DECL_FX(D)                                                                                    \
     cudaError_t fx_basis_d##D(const double *, const double *, int, void *, cudaStream_t);                  \
     size_t fx_basis_bytes_d##D(int);                                                                     \
+    cudaError_t fx_trace_d##D(const double *, const double *, int, void *, cudaStream_t);                  \
+    size_t fx_trace_bytes_d##D(int);                                                                     \
+    size_t fx_adjoint_leaf_bytes_d##D();                                                                  \
     size_t fx_leaf_bytes_d##D();
 PM_DECL_FX(8)
 PM_DECL_FX(16)
@@ -106,7 +109,9 @@ struct parament_ctx {
     Workspace hraw, full, packed64, packed32, bnorm, partials, tickets, counters, status, check;
     Workspace ctrl_copy, ctrl_conv, uout, bmax, cpacked64, cpacked32, cbnorm;
     Workspace gv, gvdag, gleaf, gblock, gbpin, gpin, gz, gpbuf, gckpt, ggrad, lscratch, gadj;
-    Workspace fxbasis, fxg;  // FP64 digit path: basis digits, packed exponents per leaf
+    // FP64 digit path: basis digits, packed exponents per leaf; gradient: trace digits, workspace per leaf
+    Workspace fxbasis, fxg, fxtrace, fxadj;
+    bool fxtrace_ready = false;  // the trace digits belong to the current Hamiltonians
     Workspace tstage, tpsi;  // trajectory: staging of a host output, psi_0 padded (FP64)
     std::vector<double2> tpsi_host;
     // batched plan
@@ -840,7 +845,8 @@ int parament_destroy(parament_ctx *ctx) {
                             &ctx->gadj,
                             &ctx->bparams, &ctx->binsts, &ctx->btable, &ctx->bitems, &ctx->bfull, &ctx->bpacked,
                             &ctx->bnorms, &ctx->bpartials, &ctx->btickets, &ctx->bcounters, &ctx->bstatus,
-                            &ctx->bqueue, &ctx->bscratch, &ctx->cheb, &ctx->tstage, &ctx->tpsi, &ctx->fxbasis, &ctx->fxg};
+                            &ctx->bqueue, &ctx->bscratch, &ctx->cheb, &ctx->tstage, &ctx->tpsi, &ctx->fxbasis, &ctx->fxg,
+                            &ctx->fxtrace, &ctx->fxadj};
         if (ctx->b_exec) cudaGraphExecDestroy(ctx->b_exec);
         for (Workspace *w : all) ws_free(*w);
     }
@@ -951,6 +957,7 @@ int parament_set_hamiltonians(parament_ctx *ctx, int dim, int n_ctrl, const void
                                                       kept, ctx->fxbasis.ptr, ctx->stream));
     }
     ctx->nb_eff = kept;
+    ctx->fxtrace_ready = false;
 
     ctx->dim = dim;
     ctx->dpad = Dp;
@@ -1148,6 +1155,27 @@ __global__ void vdag_kernel(const InT *V, int d, int Dp, double2 *out, double *z
         out[t] = v;
     }
     if (threadIdx.x == 0) z[3] = 0.0;
+    if (d > 16) return;  // vnorm_kernel follows
+    // the same bound here: thread 16 i + j forms (V^dagger V)_ij
+    __shared__ double rows[16];
+    __syncthreads();
+    const int i = threadIdx.x >> 4, j = threadIdx.x & 15;
+    double re = 0.0, im = 0.0;
+    if (i < d && j < d)
+        for (int k = 0; k < d; ++k) {
+            const double2 a = out[i * Dp + k], b = out[j * Dp + k];
+            re = fma(a.x, b.x, fma(a.y, b.y, re));
+            im = fma(a.y, b.x, fma(-a.x, b.y, im));
+        }
+    double s = sqrt(re * re + im * im);
+    for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (j == 0) rows[i] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double m = 0.0;
+        for (int r = 0; r < d; ++r) m = rows[r] > m || isnan(rows[r]) ? rows[r] : m;
+        z[3] = m;
+    }
 }
 
 // z[3] = max_i sum_j |(V^dagger V)_ij| >= ||V||_2^2 (one for a unitary V): bounds the matrices of the adjoint sweep,
@@ -1321,7 +1349,7 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     } else {
         if ((st = ws_reserve(ctx, ctx->gblock, (size_t)grid * DD * sizeof(double2)))) return st;
         if ((st = ws_reserve(ctx, ctx->gbpin, 2 * (size_t)grid * DD * sizeof(double2)))) return st;
-        if ((st = ws_reserve(ctx, ctx->gpin, 2 * (size_t)L * DD * sizeof(double2)))) return st;
+        if ((st = ws_reserve(ctx, ctx->gpin, (2 * (size_t)L + 1) * DD * sizeof(double2)))) return st;
         p.block_out = (double2 *)ctx->gblock.ptr;
         PM_CUDA(fused_dispatch(Dp, fp64, (int)ctx->integ, p, grid, warps, smem, ctx->stream));
         record_launch(ctx, ctx->nb_eff, grid, warps, lpb);
@@ -1331,7 +1359,19 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     int aw = 8, agrid = 0;
     size_t asmem = 0;
     int64_t TG = 0;
-    if (large) {
+    const bool fx_adjoint = fp64 && (Dp == 8 || Dp == 16);  // one warp per leaf on the digit products, one sweep
+    if (fx_adjoint) {
+        asmem = ctx->smem_optin;
+        if ((st = ws_reserve(ctx, ctx->fxadj, (size_t)L * (Dp == 8 ? fx_adjoint_leaf_bytes_d8() : fx_adjoint_leaf_bytes_d16()))))
+            return st;
+        if (!ctx->fxtrace_ready) {
+            const int nb = ctx->nb_eff;
+            if ((st = ws_reserve(ctx, ctx->fxtrace, Dp == 8 ? fx_trace_bytes_d8(nb) : fx_trace_bytes_d16(nb)))) return st;
+            PM_CUDA((Dp == 8 ? fx_trace_d8 : fx_trace_d16)((const double *)ctx->cpacked64.ptr,
+                                                          (const double *)ctx->cbnorm.ptr, nb, ctx->fxtrace.ptr, ctx->stream));
+            ctx->fxtrace_ready = true;
+        }
+    } else if (large) {
         asmem = adjoint_large_smem(Dp, fp64);
         if (asmem > ctx->smem_optin)
             return set_err(ctx, PARAMENT_ERR_UNSUPPORTED, "adjoint needs %zu B shared memory", asmem);
@@ -1352,8 +1392,10 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     const size_t cap = (size_t)ctx->opt_workspace_mb << 20;
     while (c_sub > 1 && (size_t)TG * c_sub * DD * csz > cap) c_sub = (c_sub + 1) / 2;
     const int64_t n_ckpt = std::max<int64_t>(1, (maxlen + c_sub - 1) / c_sub);
-    if ((st = ws_reserve(ctx, ctx->gpbuf, (size_t)TG * c_sub * DD * csz))) return st;
-    if ((st = ws_reserve(ctx, ctx->gckpt, (size_t)TG * n_ckpt * DD * csz))) return st;
+    if (!fx_adjoint) {
+        if ((st = ws_reserve(ctx, ctx->gpbuf, (size_t)TG * c_sub * DD * csz))) return st;
+        if ((st = ws_reserve(ctx, ctx->gckpt, (size_t)TG * n_ckpt * DD * csz))) return st;
+    }
     if (large && (st = ws_reserve(ctx, ctx->gadj, (size_t)L * kGradSlots * DD * csz))) return st;
 
     void *gdst = grad_out;
@@ -1373,7 +1415,7 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     sp.bpin = (double2 *)ctx->gbpin.ptr;
     sp.bsout = sp.bpin + (size_t)grid * DD;
     sp.pin = (double2 *)ctx->gpin.ptr;
-    sp.sout = sp.pin + (size_t)L * DD;
+    sp.sout = sp.pin + (size_t)(L + 1) * DD;
     sp.vdag = (const double2 *)ctx->gvdag.ptr;
     sp.z = (double *)ctx->gz.ptr;
     sp.U_out = nullptr;
@@ -1403,6 +1445,9 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     gp.n_leaves = L;
     gp.d_true = d;
     gp.status = (unsigned *)ctx->status.ptr;
+    gp.fx_basis = ctx->fxbasis.ptr;
+    gp.fx_trace = ctx->fxtrace.ptr;
+    gp.fx_g = ctx->fxadj.ptr;
     {
         const double u = fp64 ? std::ldexp(1.0, -53) : std::ldexp(1.0, -24);
         FusedParams tmp;
@@ -1527,7 +1572,7 @@ int parament_propagate_trajectory(parament_ctx *ctx, const void *psi0, void *out
     }
     if ((st = ws_reserve(ctx, ctx->gblock, (size_t)grid * DD * sizeof(double2)))) return st;
     if ((st = ws_reserve(ctx, ctx->gbpin, 2 * (size_t)grid * DD * sizeof(double2)))) return st;
-    if ((st = ws_reserve(ctx, ctx->gpin, 2 * (size_t)L * DD * sizeof(double2)))) return st;
+    if ((st = ws_reserve(ctx, ctx->gpin, (2 * (size_t)L + 1) * DD * sizeof(double2)))) return st;
     p.leaf_out = (double2 *)ctx->gleaf.ptr;
     p.block_out = (double2 *)ctx->gblock.ptr;
     PM_CUDA(fused_dispatch(Dp, fp64, (int)ctx->integ, p, grid, warps, smem, ctx->stream));
@@ -1543,7 +1588,7 @@ int parament_propagate_trajectory(parament_ctx *ctx, const void *psi0, void *out
     sp.bpin = (double2 *)ctx->gbpin.ptr;
     sp.bsout = sp.bpin + (size_t)grid * DD;
     sp.pin = (double2 *)ctx->gpin.ptr;
-    sp.sout = sp.pin + (size_t)L * DD;
+    sp.sout = sp.pin + (size_t)(L + 1) * DD;
     sp.d_out = d;
     PM_CUDA(scan_run(Dp, sp, ctx->stream));
 

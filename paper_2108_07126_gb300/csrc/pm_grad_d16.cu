@@ -1,5 +1,5 @@
 // Instantiations of the gradient kernels for padded dimension 16.
-#include "pm_grad.cuh"
+#include "pm_fx_grad.cuh"
 
 namespace pm {
 
@@ -21,47 +21,44 @@ static int adjoint_occupancy(int warps, size_t smem) {
     return e == cudaSuccess ? nb : 0;
 }
 
+// scans, then the adjoint: FP32 by groups of lanes on the CUDA cores, FP64 by the digit products (smem: the shared
+// memory limit of a block there)
 cudaError_t grad_run_d16(int fp64, int integ, const ScanParams &sp, const GradParams &gp, int grid, int warps,
                          size_t smem, cudaStream_t st) {
-    scan_blocks_kernel<16><<<1, 256, 0, st>>>(sp);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = fx::scan_run<16>(sp, sp.bpin, true, st);
     if (e != cudaSuccess) return e;
-    scan_leaves_kernel<16><<<sp.n_blocks, 256, 0, st>>>(sp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     switch (integ * 2 + (fp64 ? 1 : 0)) {
         case 0: return adjoint_launch<float, kMidpoint>(gp, grid, warps, smem, st);
-        case 1: return adjoint_launch<double, kMidpoint>(gp, grid, warps, smem, st);
+        case 1: return fx::adjoint_launch<16, kMidpoint>(gp, smem, st);
         case 2: return adjoint_launch<float, kGL2>(gp, grid, warps, smem, st);
-        case 3: return adjoint_launch<double, kGL2>(gp, grid, warps, smem, st);
+        case 3: return fx::adjoint_launch<16, kGL2>(gp, smem, st);
         case 4: return adjoint_launch<float, kSimpson>(gp, grid, warps, smem, st);
-        case 5: return adjoint_launch<double, kSimpson>(gp, grid, warps, smem, st);
+        case 5: return fx::adjoint_launch<16, kSimpson>(gp, smem, st);
     }
     return cudaErrorInvalidValue;
 }
 
-// exclusive prefixes and suffixes of every leaf from the forward pass's leaf and block products
-cudaError_t scan_run_d16(const ScanParams &sp, cudaStream_t st) {
-    scan_blocks_kernel<16><<<1, 256, 0, st>>>(sp);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    scan_leaves_kernel<16><<<sp.n_blocks, 256, 0, st>>>(sp);
-    return cudaGetLastError();
+// exclusive prefixes of every leaf from the forward pass's leaf and block products
+cudaError_t scan_run_d16(const ScanParams &sp, cudaStream_t st) { return fx::scan_run<16>(sp, sp.bpin, false, st); }
+
+cudaError_t fx_trace_d16(const double *packed, const double *bnorm, int nb, void *out, cudaStream_t st) {
+    return fx::trace_digits<16>(packed, bnorm, nb, out, st);
 }
+size_t fx_trace_bytes_d16(int nb) { return fx::trace_digit_bytes<16>(nb); }
+size_t fx_adjoint_leaf_bytes_d16() { return fx::AdjCfg<16>::LEAF_BYTES; }
 
 int adjoint_blocks_per_sm_d16(int fp64, int integ, int warps, size_t smem) {
     switch (integ * 2 + (fp64 ? 1 : 0)) {
         case 0: return adjoint_occupancy<float, kMidpoint>(warps, smem);
-        case 1: return adjoint_occupancy<double, kMidpoint>(warps, smem);
         case 2: return adjoint_occupancy<float, kGL2>(warps, smem);
-        case 3: return adjoint_occupancy<double, kGL2>(warps, smem);
         case 4: return adjoint_occupancy<float, kSimpson>(warps, smem);
-        case 5: return adjoint_occupancy<double, kSimpson>(warps, smem);
     }
     return 0;
 }
 
 size_t adjoint_smem_d16(int fp64, int K, int warps) {
-    return fp64 ? adjoint_smem_bytes<double, 16>(K, warps) : adjoint_smem_bytes<float, 16>(K, warps);
+    (void)fp64;  // FP64: sized by its own launch (pm_fx_grad.cuh)
+    return adjoint_smem_bytes<float, 16>(K, warps);
 }
 
 }  // namespace pm
