@@ -1015,7 +1015,7 @@ namespace {
 // Controls in the compute type, Taylor table and launch geometry of the fused
 // forward kernel (shared by propagate and propagate_grad).
 int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int &grid, int &warps, size_t &smem,
-                  int &leaves_per_block, int tc = 0, int cheb = 0) {
+                  int &leaves_per_block, int tc = 0, int cheb = 0, bool only_u = false) {
     const int Dp = ctx->dpad, nb = ctx->nb_eff;
     const void *ctrl = ctx->ctrl;
     const int64_t count = (int64_t)ctx->K * ctx->S;
@@ -1061,6 +1061,11 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
     } else {
     const int max_warps = fused_max_warps(Dp, fp64, cheb);
     warps = (int)ctx->opt_warps;
+    const bool su2 = Dp == 2 && only_u;  // U(T) of a two-level system: one thread per leaf (pm_su2.cuh)
+    if (warps <= 0 && su2) {
+        // one block up to 256 slices (no tree between blocks), else blocks of 128 threads
+        warps = ctx->n_steps <= 256 ? (int)std::max<int64_t>(1, (ctx->n_steps + 31) / 32) : 4;
+    }
     if (warps <= 0) {
         warps = max_warps;
         while (warps > 1 && fused_smem(Dp, fp64, nb, warps, cheb) > ctx->smem_optin) --warps;
@@ -1085,6 +1090,12 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
     if (bps <= 0) return set_err(ctx, PARAMENT_ERR_CUDA, "occupancy query failed (%d warps, %zu B)", warps, smem);
     leaves_per_block = warps * fused_gpw(Dp, fp64, cheb);
     grid = (int)ctx->opt_grid;
+    if (grid <= 0 && su2) {
+        // one slice per thread while the grid holds them (a slice costs more than a step of the product tree); the
+        // FP64 pipe is full with 4 blocks per SM, the FP32 pipe takes 8
+        const int64_t need = (ctx->n_steps + leaves_per_block - 1) / leaves_per_block;
+        grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)(fp64 ? 4 : 8) * ctx->sm_count));
+    }
     if (grid <= 0) {
         const int lm = fp64 ? kLeafMinSteps64 : kLeafMinSteps;
         const int64_t need = (ctx->n_steps + (int64_t)leaves_per_block * lm - 1) / ((int64_t)leaves_per_block * lm);
@@ -1240,7 +1251,7 @@ int parament_propagate(parament_ctx *ctx, void *U_out, parament_precision prec) 
     int grid = 0, warps = 0, lpb = 0;
     size_t smem = 0;
     const int cheb = ctx->opt_exp_method == 1;
-    int st = forward_setup(ctx, fp64, dst, p, grid, warps, smem, lpb, tc, cheb);
+    int st = forward_setup(ctx, fp64, dst, p, grid, warps, smem, lpb, tc, cheb, !cheb);
     if (st) return st;
     if (cheb) {
         // common spectral half-width over all slices, then degree and coefficients, on the device

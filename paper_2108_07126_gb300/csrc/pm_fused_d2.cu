@@ -1,11 +1,24 @@
 // Instantiations of the fused propagation kernel for padded dimension 2
 // (mode cheb: 0 = Taylor exponential, 1 = Chebyshev exponential, 2 = Taylor trajectory).
 #include "pm_fused.cuh"
+#include "pm_su2.cuh"
 
 namespace pm {
 
 cudaError_t fused_dispatch_d2(int fp64, int integ, const FusedParams &p, int grid, int warps, size_t smem,
                                cudaStream_t st, int cheb) {
+    // U(T) alone: unit quaternions, one thread per leaf (a leaf per lane in the fused kernel too, so that the caller's
+    // geometry holds for both); the fused kernel where leaf or block products are kept
+    if (cheb == 0 && !p.leaf_out && !p.block_out) {
+        switch (integ * 2 + (fp64 ? 1 : 0)) {
+            case 0: return su2::launch<float, kMidpoint>(p, grid, warps, st);
+            case 1: return su2::launch<double, kMidpoint>(p, grid, warps, st);
+            case 2: return su2::launch<float, kGL2>(p, grid, warps, st);
+            case 3: return su2::launch<double, kGL2>(p, grid, warps, st);
+            case 4: return su2::launch<float, kSimpson>(p, grid, warps, st);
+            case 5: return su2::launch<double, kSimpson>(p, grid, warps, st);
+        }
+    }
     switch (cheb * 6 + integ * 2 + (fp64 ? 1 : 0)) {
         case 0: return launch_fused<float, 2, kMidpoint>(p, grid, warps, smem, st);
         case 1: return launch_fused<double, 2, kMidpoint>(p, grid, warps, smem, st);

@@ -82,14 +82,14 @@ __device__ __forceinline__ void cos_sinc(double r2, double &c, double &s) {
 __device__ __forceinline__ void cos_sinc(float r2, float &c, float &s) {
     c = fma(r2, -1.f / 3628800.f, 1.f / 40320.f);
     s = fma(r2, -1.f / 39916800.f, 1.f / 362880.f);
-    c = fma(r2, -(-c), -1.f / 720.f);
-    s = fma(r2, -(-s), -1.f / 5040.f);
-    c = fma(r2, c, 1.f / 24.f);
-    s = fma(r2, s, 1.f / 120.f);
-    c = fma(r2, c, -0.5f);
-    s = fma(r2, s, -1.f / 6.f);
-    c = fma(r2, c, 1.f);
-    s = fma(r2, s, 1.f);
+    c = fma(r2, -c, 1.f / 720.f);
+    s = fma(r2, -s, 1.f / 5040.f);
+    c = fma(r2, -c, 1.f / 24.f);
+    s = fma(r2, -s, 1.f / 120.f);
+    c = fma(r2, -c, 0.5f);
+    s = fma(r2, -s, 1.f / 6.f);
+    c = fma(r2, -c, 1.f);
+    s = fma(r2, -s, 1.f);
 }
 
 constexpr int kMaxWarps = 8;
