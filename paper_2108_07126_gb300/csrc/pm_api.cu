@@ -1846,11 +1846,15 @@ int batch_run(parament_ctx *ctx, const parament_instance *inst, int n, parament_
         if (cls >= 0 && !((cuda_mask >> cls) & 1u)) needs_tc = true;
     }
     const int variant = (magnus ? 4 : 0) + (fp64 ? 3 : (needs_tc ? tc : 0));
-    const int leaf_steps = ctx->opt_batch_leaf > 0 ? (int)ctx->opt_batch_leaf : 64;
+    // slices per leaf: the option, or by dimension -- a leaf is a serial chain, and 64 slices of a 64 x 64 system take
+    // 1.7 ms (the end of the batch waits for the last ones), of a 2 x 2 system 30 us
+    auto leaf_steps_of = [&](int D) {
+        return ctx->opt_batch_leaf > 0 ? (int)ctx->opt_batch_leaf : (D >= 32 ? 8 : (D == 16 ? 16 : 64));
+    };
     const int items_per_sm = ctx->opt_batch_items > 0 ? (int)ctx->opt_batch_items : 32;
     const size_t csz = fp64 ? 16 : 8, rsz = fp64 ? 8 : 4;
 
-    std::vector<int64_t> key = {n, dtype, cdtype, integ, prec, leaf_steps, items_per_sm, (int64_t)cuda_mask};
+    std::vector<int64_t> key = {n, dtype, cdtype, integ, prec, ctx->opt_batch_leaf, items_per_sm, (int64_t)cuda_mask};
     for (int i = 0; i < n; ++i) {
         key.push_back(inst[i].dim);
         key.push_back(inst[i].n_ctrl);
@@ -1885,10 +1889,10 @@ int batch_run(parament_ctx *ctx, const parament_instance *inst, int n, parament_
                 int w = 8;
                 while (w > 1 && fused_smem(Dp[i], fp64, nbs[i], w, 1) > ctx->smem_optin) --w;
                 warps_of[i] = w;
-                nb_cap = std::max<int64_t>(1, N / ((int64_t)w * fused_gpw(Dp[i], fp64, 1) * leaf_steps));
+                nb_cap = std::max<int64_t>(1, N / ((int64_t)w * fused_gpw(Dp[i], fp64, 1) * leaf_steps_of(Dp[i])));
                 smem = std::max(smem, fused_smem(Dp[i], fp64, nbs[i], w, 1));
             } else {
-                nb_cap = std::max<int64_t>(1, N / leaf_steps);
+                nb_cap = std::max<int64_t>(1, N / leaf_steps_of(Dp[i]));
                 const int cls = batch_tc_class(Dp[i]);
                 const bool on_tc = tc && cls >= 0 && !((cuda_mask >> cls) & 1u);
                 smem = std::max(smem, large_smem(Dp[i], fp64, nbs[i], on_tc ? tc : 0));

@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "pm_common.cuh"
+#include "pm_digits.cuh"
 #include "pm_pp16.cuh"
 
 namespace pm {
@@ -906,20 +907,77 @@ __device__ __forceinline__ void fused_body(const FusedParams &p, int blk, int nb
             __threadfence();
             const double2 *gL = p.partials + (size_t)((idx & ~1) << level) * DD;
             const double2 *gR = p.partials + (size_t)((idx | 1) << level) * DD;
-            for (int t = tid; t < DD; t += blockDim.x) {
-                bufL[(t / D) * GD::LD + t % D] = __ldcg(gL + t);
-                bufR[(t / D) * GD::LD + t % D] = __ldcg(gR + t);
-            }
-            __syncthreads();
-            if (warp == 0 && lane < GD::LANES) {
-                double2 acc[GD::TR][GD::TC];
-                mm_tile<double, D>(bufR, bufL, rb64, cb64, acc);
-                double2 *dst = p.partials + (size_t)((idx & ~1) << level) * DD;
+            if constexpr (D >= 8) {
+                // exact digit products on the tensor cores (pm_digits.cuh): D = 16 takes one warp 9.7 k cycles on the
+                // FP64 pipe, here four warps about 1 k (a quarter of the output each; fewer warps take turns)
+                constexpr int NQ = D == 16 ? 4 : 1;
+                uint32_t *rhs = (uint32_t *)wbase;
+                static_assert(fx::rhs_words<D>() * 4 <= GPW * G::GSTRIDE, "a right operand fits in a warp's slots");
+                long long o[NQ][4];
+                bool bad = false;
 #pragma unroll
-                for (int r = 0; r < GD::TR; ++r)
+                for (int k = 0; k < NQ; ++k) {
+                    const int qt = warp + k * W;
+                    if (!active_warp || qt >= NQ) continue;
+                    fx::Tile<D> t;
+                    fx::Digits<D> d;
 #pragma unroll
-                    for (int c = 0; c < GD::TC; ++c)
-                        __stcg(dst + (rb64 + r * GD::RBN) * D + GD::col(cb64, c), acc[r][c]);
+                    for (int e = 0; e < fx::L<D>::NE; ++e) {
+                        const double2 v = __ldcg(gL + fx::L<D>::col(lane, e) * D + fx::L<D>::row(lane, e));
+                        bad |= !(fabs(v.x) < 2.0) || !(fabs(v.y) < 2.0);
+                        t.re[e] = fx::from_double(v.x, 0);
+                        t.im[e] = fx::from_double(v.y, 0);
+                    }
+                    fx::split<D>(t, d);
+                    fx::put_rhs<D>(rhs, lane, d, fx::kPlain);
+#pragma unroll
+                    for (int e = 0; e < fx::L<D>::NE; ++e) {
+                        const double2 v = __ldcg(gR + fx::L<D>::row(lane, e) * D + fx::L<D>::col(lane, e));
+                        bad |= !(fabs(v.x) < 2.0) || !(fabs(v.y) < 2.0);
+                        t.re[e] = fx::from_double(v.x, 0);
+                        t.im[e] = fx::from_double(v.y, 0);
+                    }
+                    fx::split<D>(t, d);
+                    if constexpr (D == 16) {
+                        fx::mul16_quarter(d, rhs, lane, qt >> 1, qt & 1, o[k]);
+                    } else {
+                        fx::mul(d, rhs, lane, t);
+                        o[k][0] = t.re[0];
+                        o[k][1] = t.re[1];
+                        o[k][2] = t.im[0];
+                        o[k][3] = t.im[1];
+                    }
+                }
+                const double nanv = __syncthreads_or(bad) ? nan("") : 0.0;  // every factor is read
+                double *dst = (double *)(p.partials + (size_t)((idx & ~1) << level) * DD);
+#pragma unroll
+                for (int k = 0; k < NQ; ++k) {
+                    const int qt = warp + k * W;
+                    if (!active_warp || qt >= NQ) continue;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = (lane >> 2) + (D == 16 ? 8 * (u >> 1) : 0);
+                        const int j = (D == 16 ? 8 * (qt >> 1) : 0) + 2 * (lane & 3) + (u & 1);
+                        const int part = D == 16 ? (qt & 1) : (u >> 1);
+                        __stcg(dst + 2 * (i * D + j) + part, fx::to_double(o[k][u]) + nanv);
+                    }
+                }
+            } else {
+                for (int t = tid; t < DD; t += blockDim.x) {
+                    bufL[(t / D) * GD::LD + t % D] = __ldcg(gL + t);
+                    bufR[(t / D) * GD::LD + t % D] = __ldcg(gR + t);
+                }
+                __syncthreads();
+                if (warp == 0 && lane < GD::LANES) {
+                    double2 acc[GD::TR][GD::TC];
+                    mm_tile<double, D>(bufR, bufL, rb64, cb64, acc);
+                    double2 *dst = p.partials + (size_t)((idx & ~1) << level) * DD;
+#pragma unroll
+                    for (int r = 0; r < GD::TR; ++r)
+#pragma unroll
+                        for (int c = 0; c < GD::TC; ++c)
+                            __stcg(dst + (rb64 + r * GD::RBN) * D + GD::col(cb64, c), acc[r][c]);
+                }
             }
             __threadfence();
             __syncthreads();
