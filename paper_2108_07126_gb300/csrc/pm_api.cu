@@ -51,7 +51,7 @@ PM_DECL_FX(16)
     cudaError_t large_dispatch_d##D(int, int, const FusedParams &, void *, int, size_t, cudaStream_t, int); \
     int large_blocks_per_sm_d##D(int, int, size_t, int);                                                 \
     size_t large_smem_d##D(int, int, int);                                                               \
-    cudaError_t large_prefix_d##D(const double2 *, int, double2 *, double2 *, double2 **, cudaStream_t);    \
+    cudaError_t large_prefix_d##D(const double2 *, int, int, double2 *, double2 *, double2 **, cudaStream_t);    \
     cudaError_t grad_large_run_d##D(int, int, const double2 *, int, double2 *, double2 *, const GradParams &, \
                                     void *, void *, int, int, cudaStream_t);                             \
     size_t adjoint_large_smem_d##D(int);
@@ -649,12 +649,12 @@ size_t adjoint_large_smem(int Dp, int fp64) {
     }
     return 0;
 }
-cudaError_t large_prefix(int Dp, const double2 *leaf, int n, double2 *a, double2 *b, double2 **x, cudaStream_t st) {
+cudaError_t large_prefix(int Dp, const double2 *leaf, int n, int d, double2 *a, double2 *b, double2 **x, cudaStream_t st) {
     switch (Dp) {
-        case 32: return large_prefix_d32(leaf, n, a, b, x, st);
-        case 64: return large_prefix_d64(leaf, n, a, b, x, st);
-        case 128: return large_prefix_d128(leaf, n, a, b, x, st);
-        case 256: return large_prefix_d256(leaf, n, a, b, x, st);
+        case 32: return large_prefix_d32(leaf, n, d, a, b, x, st);
+        case 64: return large_prefix_d64(leaf, n, d, a, b, x, st);
+        case 128: return large_prefix_d128(leaf, n, d, a, b, x, st);
+        case 256: return large_prefix_d256(leaf, n, d, a, b, x, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -1566,7 +1566,7 @@ int parament_propagate_trajectory(parament_ctx *ctx, const void *psi0, void *out
         PM_CUDA(forward_launch(ctx, fp64, p, grid, warps, smem));
         record_launch(ctx, ctx->nb_eff, grid, warps, lpb);
         double2 *pin = nullptr;
-        PM_CUDA(large_prefix(Dp, (const double2 *)ctx->gleaf.ptr, (int)L, (double2 *)ctx->gpin.ptr,
+        PM_CUDA(large_prefix(Dp, (const double2 *)ctx->gleaf.ptr, (int)L, d, (double2 *)ctx->gpin.ptr,
                              (double2 *)ctx->gpin.ptr + (size_t)L * DD, &pin, ctx->stream));
         FusedParams pt = p;
         pt.leaf_out = nullptr;

@@ -45,15 +45,17 @@ __device__ __forceinline__ i64 to_fixed(double v, bool &bad) {
     return (i64)b < 0 ? -(i64)q : (i64)q;
 }
 
-// C = A B for one BM x BM block: A is BM x K (row stride lda), B is K x BM (ldb), C (ldc) must not alias them.
-// All 256 threads; smem: G<BM>::BYTES.  Starts after the caller's barrier and ends with one.
+// C = A B for one block of at most BM x BM: A is rows x K (row stride lda), B is K x cols (ldb), C (ldc) must not
+// alias them; rows, cols and K are multiples of 16 (BM = 32: rows and cols full).  All 256 threads; smem:
+// G<BM>::BYTES.  Starts after the caller's barrier and ends with one.
 template <int BM>
 __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double2 *B, int ldb, double2 *C, int ldc, int K,
-                                         unsigned char *smem) {
+                                         unsigned char *smem, int rows = BM, int cols = BM) {
     using g = G<BM>;
     constexpr int NTW = g::NTW;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rb = warp % g::RB, cw = warp / g::RB;
+    const int nrb = BM == 32 ? g::RB : rows / 16, ntw = BM == 32 ? NTW : cols / 16;  // active row blocks, tiles per warp
     uint32_t *st = (uint32_t *)smem;
     bool bad = false;
 
@@ -64,6 +66,7 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
 #pragma unroll
         for (int i = 0; i < g::IA; ++i) {
             const int w = tid + kThreads * i, l2 = (w & 127) >> 2, reg = w & 3;
+            if ((w >> 7) >= nrb) continue;
             const int r = 16 * (w >> 7) + (l2 >> 2) + 8 * (reg & 1), k = k0 + 2 * (l2 & 3) + 8 * (reg >> 1);
             va[i][0] = A[(size_t)r * lda + k];
             va[i][1] = A[(size_t)r * lda + k + 1];
@@ -71,6 +74,7 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
 #pragma unroll
         for (int i = 0; i < g::IB; ++i) {
             const int w = tid + kThreads * i, l2 = (w & 63) >> 1, reg = w & 1;
+            if ((w >> 6) >= g::WC * ntw) continue;
             const int n = 8 * (w >> 6) + (l2 >> 2), k = k0 + 2 * (l2 & 3) + 8 * reg;
             vb[i][0] = B[(size_t)k * ldb + n];
             vb[i][1] = B[(size_t)(k + 1) * ldb + n];
@@ -85,17 +89,15 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
 #pragma unroll
         for (int i = 0; i < ND; ++i) s[(2 * i + 1) * stride] = d[i];
     };
-    auto store = [&](int buf) {
+    // piece k of a panel: the thread's k-th pair of A, then of B
+    constexpr int PIECES = g::IA + g::IB;
+    auto store_piece = [&](int buf, int k) {
         uint32_t *sa = st + buf * (g::AW + g::BW), *sb = sa + g::AW;
-#pragma unroll
-        for (int i = 0; i < g::IA; ++i) {
-            const int w = tid + kThreads * i;
-            put(sa + (w >> 7) * (2 * ND * 128) + (w & 127), 128, va[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < g::IB; ++i) {
-            const int w = tid + kThreads * i;
-            put(sb + (w >> 6) * (2 * ND * 64) + (w & 63), 64, vb[i]);
+        const int w = tid + kThreads * (k < g::IA ? k : k - g::IA);
+        if (k < g::IA) {
+            if ((w >> 7) < nrb) put(sa + (w >> 7) * (2 * ND * 128) + (w & 127), 128, va[k < g::IA ? k : 0]);
+        } else if ((w >> 6) < g::WC * ntw) {
+            put(sb + (w >> 6) * (2 * ND * 64) + (w & 63), 64, vb[k < g::IA ? 0 : k - g::IA]);
         }
     };
 
@@ -108,7 +110,8 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
             for (int u = 0; u < 4; ++u) o[t][pt][u] = 0;
 
     load(0);
-    store(0);
+#pragma unroll
+    for (int k = 0; k < PIECES; ++k) store_piece(0, k);
     bool any = __syncthreads_or(bad);
     for (int kp = 0; kp < K / KP; ++kp) {
         const bool more = kp + 1 < K / KP;
@@ -124,7 +127,13 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
         }
 #pragma unroll
         for (int t = 0; t < NTW; ++t) {
-            const uint32_t *sn = sb + (cw * NTW + t) * (2 * ND * 64) + lane * 2;
+            // the next panel is converted and stored piece by piece between the tiles, beside the MMAs
+            if (more) {
+#pragma unroll
+                for (int k = t * PIECES / NTW; k < (t + 1) * PIECES / NTW; ++k) store_piece((kp + 1) & 1, k);
+            }
+            if (t >= ntw || rb >= nrb) continue;
+            const uint32_t *sn = sb + (cw * ntw + t) * (2 * ND * 64) + lane * 2;
 #pragma unroll
             for (int pt = 0; pt < 2; ++pt) {  // Re: Ar Br + Ai (-Bi); Im: Ar Bi + Ai Br
                 float acc[fx::NA][4];
@@ -155,7 +164,6 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
                 for (int u = 0; u < 4; ++u) o[t][pt][u] += fx::collect_fine(acc, u);
             }
         }
-        if (more) store((kp + 1) & 1);
         any = __syncthreads_or(bad) || any;
     }
     const double nanv = any ? nan("") : 0.0;
@@ -163,7 +171,8 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
     for (int t = 0; t < NTW; ++t)
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int r = 16 * rb + (lane >> 2) + 8 * (u >> 1), c = 8 * (cw * NTW + t) + 2 * (lane & 3) + (u & 1);
+            if (t >= ntw || rb >= nrb) continue;
+            const int r = 16 * rb + (lane >> 2) + 8 * (u >> 1), c = 8 * (cw * ntw + t) + 2 * (lane & 3) + (u & 1);
             double2 v = make_double2(fx::to_double<fx::FC>(o[t][0][u]), fx::to_double<fx::FC>(o[t][1][u]));
             if (any) v = make_double2(nanv, nanv);
             C[(size_t)r * ldc + c] = v;
@@ -171,14 +180,18 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
     __syncthreads();
 }
 
-// C = A B for D x D matrices by the whole block (256 threads); C must not alias A or B; ends with a barrier
-template <int D> __device__ __noinline__ void cta_mm(const double2 *A, const double2 *B, double2 *C, unsigned char *smem) {
-    constexpr int BM = block_of<D>(), NBK = D / BM;
+// C = A B for D x D matrices (row stride D) of true dimension d by the whole block (256 threads); C must not alias A
+// or B; ends with a barrier.  Only the leading ceil(d / 16) * 16 rows, columns and k are read and written: d = 40 in
+// its 64 x 64 frame takes 3 of 4 panels on 3 of 4 row blocks.
+__device__ __forceinline__ int extent(int d) { return (d + 15) & ~15; }
+template <int D> __device__ __noinline__ void cta_mm(const double2 *A, const double2 *B, double2 *C, unsigned char *smem, int d) {
+    constexpr int BM = block_of<D>();
+    const int n = D == 32 ? 32 : extent(d);
 #pragma unroll 1
-    for (int blk = 0; blk < NBK * NBK; ++blk) {
-        const int i = (blk / NBK) * BM, j = (blk % NBK) * BM;
-        block_mm<BM>(A + (size_t)i * D, D, B + j, D, C + (size_t)i * D + j, D, D, smem);
-    }
+    for (int i = 0; i < n; i += BM)
+#pragma unroll 1
+        for (int j = 0; j < n; j += BM)
+            block_mm<BM>(A + (size_t)i * D, D, B + j, D, C + (size_t)i * D + j, D, n, smem, min(BM, n - i), min(BM, n - j));
 }
 
 }  // namespace fxl

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(256) suffix_init_kernel(const double2 *__restr
 // factor on the left), else in_i; block (tile, i) computes one 32 x 32 tile of out_i
 template <int D>
 __global__ void __launch_bounds__(256) suffix_level_kernel(const double2 *__restrict__ in, int n, int off,
-                                                           double2 *__restrict__ out) {
+                                                           double2 *__restrict__ out, int d) {
     constexpr int T = 32;
     extern __shared__ __align__(16) unsigned char smem[];
     const int ti = blockIdx.x / (D / T), tj = blockIdx.x % (D / T), i = blockIdx.y;
@@ -50,18 +50,20 @@ __global__ void __launch_bounds__(256) suffix_level_kernel(const double2 *__rest
         return;
     }
     const double2 *Lt = in + (size_t)(i + off) * DD;  // later factor (left)
-    fxl::block_mm<T>(Lt + (size_t)(ti * T) * D, D, Rt + tj * T, D, O, D, D, smem);
+    const int ext = fxl::extent(d);
+    if (ti * T < ext && tj * T < ext) fxl::block_mm<T>(Lt + (size_t)(ti * T) * D, D, Rt + tj * T, D, O, D, ext, smem);
+    else zero_tile<T, D>(O);
 }
 
 // exclusive suffixes of n leaf products into x (one of the two buffers a, b; returned)
 template <int D>
-cudaError_t leaf_suffixes(const double2 *leaf, int n, double2 *a, double2 *b, double2 **x, cudaStream_t st) {
+cudaError_t leaf_suffixes(const double2 *leaf, int n, int d, double2 *a, double2 *b, double2 **x, cudaStream_t st) {
     suffix_init_kernel<D><<<1024, 256, 0, st>>>(leaf, n, a);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = allow_block_mm_smem(suffix_level_kernel<D>);
     double2 *cur = a, *nxt = b;
     for (int off = 1; off < n && e == cudaSuccess; off <<= 1) {
-        suffix_level_kernel<D><<<dim3((D / 32) * (D / 32), n), 256, fxl::G<32>::BYTES, st>>>(cur, n, off, nxt);
+        suffix_level_kernel<D><<<dim3((D / 32) * (D / 32), n), 256, fxl::G<32>::BYTES, st>>>(cur, n, off, nxt, d);
         e = cudaGetLastError();
         double2 *t = cur;
         cur = nxt;
@@ -77,8 +79,8 @@ __global__ void __launch_bounds__(256) z_loss_kernel(const double2 *__restrict__
                                                      double *z, void *U_out, int out_c128, int d_out) {
     __shared__ double red[2][8];
     double zr = 0.0, zi = 0.0;
-    for (int e = threadIdx.x; e < D * D; e += blockDim.x) {
-        const int i = e / D, k = e % D;
+    for (int e = threadIdx.x; e < d_out * d_out; e += blockDim.x) {  // entries beyond the dimension are not defined
+        const int i = e / d_out, k = e % d_out;
         const double2 a = vdag[i * D + k], b = U[k * D + i];
         zr = fma(a.x, b.x, fma(-a.y, b.y, zr));
         zi = fma(a.x, b.y, fma(a.y, b.x, zi));
@@ -170,7 +172,7 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
     unsigned flags = 0;
 
     auto mm = [&](const C *A, const C *B, C *Cm) {  // ends with a barrier
-        if constexpr (std::is_same<Real, double>::value) fxl::cta_mm<D>(A, B, Cm, panels);
+        if constexpr (std::is_same<Real, double>::value) fxl::cta_mm<D>(A, B, Cm, panels, (int)p.d_true);
         else cta_mm<Real, D>(A, B, Cm, panels);
     };
     auto ld_glob = [&](C *S, const double2 *src) {
@@ -369,6 +371,7 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
                 Real tr = 0, ti = 0;
                 for (int el = tid; el < DD; el += NT) {
                     const int i = el / D, jj = el % D;
+                    if (i >= (int)p.d_true || jj >= (int)p.d_true) continue;  // not defined beyond the dimension
                     const Real av = __ldg(Pe + jj * D + i), bv = __ldg(Pe + i * D + jj);
                     const Real br = (jj <= i) ? av : bv;
                     const Real bi = (jj > i) ? av : ((jj < i) ? -bv : Real(0));
@@ -470,8 +473,8 @@ cudaError_t grad_large_run(int fp64, int integ, const double2 *leaf, int L, doub
                            GradParams gp, void *scratch, void *U_out, int out_c128, int d_out, cudaStream_t st) {
     const size_t DD = (size_t)D * D;
     double2 *xp = nullptr, *xs = nullptr;
-    cudaError_t e = leaf_prefixes<D>(leaf, L + 1, pre, pre + (size_t)(L + 1) * DD, &xp, st);
-    if (e == cudaSuccess) e = leaf_suffixes<D>(leaf, L, suf, suf + (size_t)L * DD, &xs, st);
+    cudaError_t e = leaf_prefixes<D>(leaf, L + 1, d_out, pre, pre + (size_t)(L + 1) * DD, &xp, st);
+    if (e == cudaSuccess) e = leaf_suffixes<D>(leaf, L, d_out, suf, suf + (size_t)L * DD, &xs, st);
     if (e != cudaSuccess) return e;
     z_loss_kernel<D><<<1, 256, 0, st>>>(xp + (size_t)L * DD, gp.vdag, (double *)gp.z, U_out, out_c128, d_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -227,7 +227,7 @@ __device__ __forceinline__ void smem_mm(const float2 *__restrict__ A, const floa
 template <typename Real, int D, int TCM>
 __device__ __forceinline__ void large_mm(const typename Cx<Real>::T *A, const typename Cx<Real>::T *B,
                                          typename Cx<Real>::T *Cout, unsigned char *panels, umma::Ctx *uc,
-                                         bool cheb = false) {
+                                         int d, bool cheb = false) {
     if constexpr ((TCM == 2 || TCM == 3) && std::is_same<Real, float>::value) {
         constexpr int F = TCM == 3 ? umma::kBF16x3 : umma::kTF32x3;
         if constexpr (D == 128) {
@@ -245,7 +245,7 @@ __device__ __forceinline__ void large_mm(const typename Cx<Real>::T *A, const ty
     } else if constexpr (std::is_same<Real, double>::value) {
         // digit products; the Clenshaw recurrence of the Chebyshev series leaves their range (|entry| < 2)
         if (cheb) cta_mm<Real, D>(A, B, Cout, panels);
-        else fxl::cta_mm<D>(A, B, Cout, panels);
+        else fxl::cta_mm<D>(A, B, Cout, panels, d);
     } else {
         cta_mm<Real, D>(A, B, Cout, panels);
     }
@@ -369,7 +369,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             }
             __syncthreads();
             for (int k = mch - 1; k >= 0; --k) {
-                large_mm<Real, D, TCM>(SX, d1, nw, panels, uc, true);
+                large_mm<Real, D, TCM>(SX, d1, nw, panels, uc, p.d_out, true);
                 const C a_k = ak[k];
                 for (int e = tid; e < DD; e += kLargeThreads) {
                     const C x = nw[e], y = d2[e];
@@ -389,7 +389,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
                 }
             }
             // leaf product R <- U_j R into P1 (U_j is in one of SX2, SX3, P0), which becomes R
-            large_mm<Real, D, TCM>(nw, SR, P1, panels, uc, true);
+            large_mm<Real, D, TCM>(nw, SR, P1, panels, uc, p.d_out, true);
             {
                 C *old = SR;
                 SR = P1;
@@ -401,8 +401,8 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             }
             continue;
         }
-        if (q >= 2) large_mm<Real, D, TCM>(SX, SX, SX2, panels, uc);
-        if (q >= 3) large_mm<Real, D, TCM>(SX2, SX, SX3, panels, uc);
+        if (q >= 2) large_mm<Real, D, TCM>(SX, SX, SX2, panels, uc, p.d_out);
+        if (q >= 3) large_mm<Real, D, TCM>(SX2, SX, SX3, panels, uc, p.d_out);
         const C *Xq = (q == 1) ? SX : ((q == 2) ? SX2 : SX3);
         // Horner over blocks with two ping-pong buffers:
         //   T = a_{q r} X^q + B_{r-1};  T <- X^q T + B_b;  B_b = sum_{l<q} a_{q b + l} X^l
@@ -411,6 +411,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             const Real a0 = coef<Real>(p, q * b);
             const Real a1 = (q >= 2) ? coef<Real>(p, q * b + 1) : Real(0);
             const Real a2 = (q >= 3) ? coef<Real>(p, q * b + 2) : Real(0);
+            const bool scaled = scale != Real(1);
             for (int e0 = tid; e0 < DD; e0 += 4 * kLargeThreads) {
                 C v[4], x1[4], x2[4];
 #pragma unroll
@@ -423,7 +424,8 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int e = e0 + u * kLargeThreads;
-                    C w = Cx<Real>::make(v[u].x * scale, v[u].y * scale);
+                    C w = v[u];
+                    if (scaled) w = Cx<Real>::make(v[u].x * scale, v[u].y * scale);
                     w.x += ((e / D) == (e % D)) ? a0 : Real(0);
                     if (q >= 2) {
                         w.x = fma(a1, x1[u].x, w.x);
@@ -441,16 +443,16 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
         C *cur = P0, *nxt = P1;
         add_block(cur, Xq, coef<Real>(p, q * rh), rh - 1);
         for (int b = rh - 2; b >= 0; --b) {
-            large_mm<Real, D, TCM>(Xq, cur, nxt, panels, uc);
+            large_mm<Real, D, TCM>(Xq, cur, nxt, panels, uc, p.d_out);
             add_block(nxt, nxt, Real(1), b);
             C *t2 = cur; cur = nxt; nxt = t2;
         }
         for (int i = 0; i < s; ++i) {
-            large_mm<Real, D, TCM>(cur, cur, nxt, panels, uc);
+            large_mm<Real, D, TCM>(cur, cur, nxt, panels, uc, p.d_out);
             C *t2 = cur; cur = nxt; nxt = t2;
         }
         // leaf product R <- U_j R into the free buffer, which becomes R; the old R slot is free
-        large_mm<Real, D, TCM>(cur, SR, nxt, panels, uc);
+        large_mm<Real, D, TCM>(cur, SR, nxt, panels, uc, p.d_out);
         {
             C *old = SR;
             SR = nxt;
@@ -507,13 +509,13 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
                 P0[e] = Cx<Real>::make(v.x, -v.y);  // R^dagger
             }
             __syncthreads();
-            large_mm<Real, D, TCM>(P0, SR, P1, panels, uc);  // R^dagger R
+            large_mm<Real, D, TCM>(P0, SR, P1, panels, uc, p.d_out);  // R^dagger R
             for (int e = tid; e < DD; e += kLargeThreads) {
                 const C v = P1[e];
                 P1[e] = Cx<Real>::make(((e / D) == (e % D) ? Real(3) : Real(0)) - v.x, -v.y);
             }
             __syncthreads();
-            large_mm<Real, D, TCM>(SR, P1, P0, panels, uc);  // R (3 I - R^dagger R)
+            large_mm<Real, D, TCM>(SR, P1, P0, panels, uc, p.d_out);  // R (3 I - R^dagger R)
             for (int e = tid; e < DD; e += kLargeThreads) {
                 const C v = P0[e];
                 SR[e] = Cx<Real>::make(Real(0.5) * v.x, Real(0.5) * v.y);
@@ -534,7 +536,10 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
     {
         double2 *dst = p.partials + (size_t)blk * DD;
         for (int e = tid; e < DD; e += kLargeThreads) {
-            const C v = SR[e];
+            C v = SR[e];
+            // the digit products leave the padding beyond the dimension undefined: the identity there
+            if (std::is_same<Real, double>::value && max(e / D, e % D) >= p.d_out)
+                v = Cx<Real>::make((e / D) == (e % D) ? Real(1) : Real(0), Real(0));
             dst[e] = make_double2((double)v.x, (double)v.y);
             if (p.leaf_out) p.leaf_out[(size_t)blk * DD + e] = dst[e];
             if (p.block_out) p.block_out[(size_t)blk * DD + e] = dst[e];
@@ -618,7 +623,7 @@ __device__ void large_arrival_tree(const FusedParams &p, void *ws_bytes, int blk
                     R2[e] = __ldcg(gR + e);
                 }
                 __syncthreads();
-                if constexpr (std::is_same<Real, double>::value || tree_on_digits<D>()) fxl::cta_mm<D>(R2, L2, gL, smem);
+                if constexpr (std::is_same<Real, double>::value || tree_on_digits<D>()) fxl::cta_mm<D>(R2, L2, gL, smem, p.d_out);
                 else cta_mm<double, D>(R2, L2, gL, smem);
             } else {
                 float2 *Lf = (float2 *)ws_bytes, *Rf = Lf + DD, *Cf = Rf + DD;
@@ -723,6 +728,11 @@ __global__ void __launch_bounds__(256) tree_level_kernel(const double2 *__restri
     }
 }
 
+template <int T, int D> __device__ __forceinline__ void zero_tile(double2 *O) {
+    for (int e = threadIdx.x; e < T * T; e += blockDim.x) O[(size_t)(e / T) * D + e % T] = make_double2(0.0, 0.0);
+    __syncthreads();
+}
+
 // The same level with FP64 products on the digit products: block (tile, pair) computes one 32 x 32 tile.
 // D = 128, one product: 16 blocks of 14 k cycles against 16 blocks of 308 k on the FP64 pipe.
 template <int D>
@@ -734,8 +744,10 @@ __global__ void __launch_bounds__(256) tree_level_fx_kernel(const double2 *__res
     const size_t DD = (size_t)D * D;
     const double2 *L = in + (size_t)(2 * pair) * DD, *R = L + DD;  // earlier, later
     double2 *O = out + (size_t)pair * DD + (size_t)(ti * T) * D + tj * T;
+    const int n = fxl::extent(p.d_out);  // rows and columns beyond the dimension's last tile are not used
     if (2 * pair + 1 < n_in) {
-        fxl::block_mm<T>(R + (size_t)(ti * T) * D, D, L + tj * T, D, O, D, D, smem);
+        if (ti * T < n && tj * T < n) fxl::block_mm<T>(R + (size_t)(ti * T) * D, D, L + tj * T, D, O, D, n, smem);
+        else zero_tile<T, D>(O);
     } else {
         for (int e = threadIdx.x; e < T * T; e += blockDim.x)
             O[(size_t)(e / T) * D + e % T] = L[(size_t)(ti * T + e / T) * D + tj * T + e % T];
@@ -774,7 +786,7 @@ __global__ void __launch_bounds__(256) prefix_init_kernel(const double2 *__restr
 // one level: block (tile, i) computes one 32 x 32 tile of out_i on the digit products (pm_fxl.cuh)
 template <int D>
 __global__ void __launch_bounds__(256) prefix_level_kernel(const double2 *__restrict__ in, int n, int off,
-                                                           double2 *__restrict__ out) {
+                                                           double2 *__restrict__ out, int d) {
     constexpr int T = 32;
     extern __shared__ __align__(16) unsigned char smem[];
     const int ti = blockIdx.x / (D / T), tj = blockIdx.x % (D / T), i = blockIdx.y;
@@ -787,7 +799,9 @@ __global__ void __launch_bounds__(256) prefix_level_kernel(const double2 *__rest
         return;
     }
     const double2 *Rt = in + (size_t)(i - off) * DD;  // earlier factor (right)
-    fxl::block_mm<T>(Lt + (size_t)(ti * T) * D, D, Rt + tj * T, D, O, D, D, smem);
+    const int ext = fxl::extent(d);
+    if (ti * T < ext && tj * T < ext) fxl::block_mm<T>(Lt + (size_t)(ti * T) * D, D, Rt + tj * T, D, O, D, ext, smem);
+    else zero_tile<T, D>(O);
 }
 
 // the kernels above use more than the default limit of dynamic shared memory
@@ -797,13 +811,13 @@ template <typename K> cudaError_t allow_block_mm_smem(K k) {
 
 // exclusive prefixes of n leaf products into x (one of the two buffers a, b; returned)
 template <int D>
-cudaError_t leaf_prefixes(const double2 *leaf, int n, double2 *a, double2 *b, double2 **x, cudaStream_t st) {
+cudaError_t leaf_prefixes(const double2 *leaf, int n, int d, double2 *a, double2 *b, double2 **x, cudaStream_t st) {
     prefix_init_kernel<D><<<1024, 256, 0, st>>>(leaf, n, a);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = allow_block_mm_smem(prefix_level_kernel<D>);
     double2 *cur = a, *nxt = b;
     for (int off = 1; off < n && e == cudaSuccess; off <<= 1) {
-        prefix_level_kernel<D><<<dim3((D / 32) * (D / 32), n), 256, fxl::G<32>::BYTES, st>>>(cur, n, off, nxt);
+        prefix_level_kernel<D><<<dim3((D / 32) * (D / 32), n), 256, fxl::G<32>::BYTES, st>>>(cur, n, off, nxt, d);
         e = cudaGetLastError();
         double2 *t = cur;
         cur = nxt;
