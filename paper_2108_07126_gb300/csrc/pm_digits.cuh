@@ -295,6 +295,53 @@ __device__ __forceinline__ void mul(const Digits<8> &a, const uint32_t *rhs, int
     o.im[1] = collect(acc, 3);
 }
 
+// o = a1 B1 + a2 B2
+__device__ __forceinline__ void mul_sum(const Digits<16> &a1, const uint32_t *rhs1, const Digits<16> &a2, const uint32_t *rhs2,
+                                        int lane, Tile<16> &o) {
+    mul(a1, rhs1, lane, o);
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            i64 v[4];
+            mul16_quarter(a2, rhs2, lane, nt, part, v);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (part) o.im[4 * nt + u] += v[u];
+                else o.re[4 * nt + u] += v[u];
+            }
+        }
+}
+// (D = 8: both products in one set of accumulators, 32 real terms as in one 16 x 16 product)
+__device__ __forceinline__ void mul_sum(const Digits<8> &a1, const uint32_t *rhs1, const Digits<8> &a2, const uint32_t *rhs2,
+                                        int lane, Tile<8> &o) {
+    float acc[NA][4];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const Digits<8> &a = k ? a2 : a1;
+        const uint32_t *rhs = k ? rhs2 : rhs1;
+        uint32_t b[ND][2];
+#pragma unroll
+        for (int j = 0; j < ND; ++j) {
+            b[j][0] = rhs[(j * 2 + 0) * 32 + lane];
+            b[j][1] = rhs[(j * 2 + 1) * 32 + lane];
+        }
+#pragma unroll
+        for (int i = 0; i < ND; ++i) {
+            const uint32_t n = neg2(a.im[i][0]);
+#pragma unroll
+            for (int j = 0; j <= last_digit(i); ++j) {
+                if (k == 0 && first_pair(i, j)) mma_first(acc[i + j], a.re[i][0], a.im[i][0], n, a.re[i][0], b[j][0], b[j][1], acc_start(i + j));
+                else mma(acc[i + j], a.re[i][0], a.im[i][0], n, a.re[i][0], b[j][0], b[j][1]);
+            }
+        }
+    }
+    o.re[0] = collect(acc, 0);
+    o.re[1] = collect(acc, 1);
+    o.im[0] = collect(acc, 2);
+    o.im[1] = collect(acc, 3);
+}
+
 // tile <-> shared memory private to the lane: entry e at e * 32 + lane (16 bytes)
 template <int D> __device__ __forceinline__ void st_priv(longlong2 *S, int lane, const Tile<D> &t) {
 #pragma unroll

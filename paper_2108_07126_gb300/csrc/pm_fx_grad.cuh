@@ -253,8 +253,8 @@ template <int D> cudaError_t scan_run(const ScanParams &sp, double2 *groups, boo
 
 template <int D> struct AdjCfg {
     static constexpr int W = D == 16 ? 8 : 16;                  // warps per block
-    static constexpr bool TILES_GLOBAL = D == 16;               // 32 KB of tiles per warp: in L2 for D = 16
-    static constexpr int NTILE = 8;                             // Y, Y^2, D1, D2, T, M, P^T, W^T
+    static constexpr bool TILES_GLOBAL = D == 16;               // 24 KB of tiles per warp: in L2 for D = 16
+    static constexpr int NTILE = 6;                             // Y, Y^2, D1, D2, P^T, W^T
     static constexpr int TILE = Cfg<D>::TILE, RHS = Cfg<D>::RHS;
     // global memory per leaf: packed exponents and M of a tile of slices, and the tiles
     static constexpr size_t LEAF_BYTES = (size_t)kGT * D * D * 8 * 3 + (TILES_GLOBAL ? (size_t)NTILE * TILE : 0);
@@ -363,8 +363,8 @@ __global__ void __launch_bounds__(AdjCfg<D>::W * 32, 1) fx_adjoint_kernel(const 
     uint32_t *r1 = (uint32_t *)wbase, *r2 = r1 + rhs_words<D>(), *r3 = r2 + rhs_words<D>();
     longlong2 *tiles = AdjCfg<D>::TILES_GLOBAL ? (longlong2 *)(mbuf + 2 * kGT * DD)
                                                : (longlong2 *)(wbase + wb - 64 - (size_t)AdjCfg<D>::NTILE * AdjCfg<D>::TILE);
-    longlong2 *SY = tiles, *SY2 = tiles + NT, *SD1 = tiles + 2 * NT, *SD2 = tiles + 3 * NT, *ST = tiles + 4 * NT,
-              *SM = tiles + 5 * NT, *SP = tiles + 6 * NT, *SW = tiles + 7 * NT;
+    longlong2 *SY = tiles, *SY2 = tiles + NT, *SD1 = tiles + 2 * NT, *SD2 = tiles + 3 * NT, *SP = tiles + 4 * NT,
+              *SW = tiles + 5 * NT;
     i64 *xpk = (i64 *)r1;  // packed exponent, before the right operands
     double *gam = (double *)wbase;  // coefficients of a tile (before its slices), traces of a tile (after them)
     int *cls = (int *)(wbase + wb - 64);
@@ -375,26 +375,10 @@ __global__ void __launch_bounds__(AdjCfg<D>::W * 32, 1) fx_adjoint_kernel(const 
     const double vn = p.z[3];
     const int ve = (vn > 1.5 && vn < 1e300) ? ilogb(vn) / 2 + 1 : 0;
 
-    auto mul_by = [&](const longlong2 *S, const uint32_t *rhs, Tile<D> &o) {  // o = S * right operand
+    auto split_of = [&](const longlong2 *S, Digits<D> &d) {
         Tile<D> t;
-        Digits<D> d;
         ld_priv<D>(S, lane, t);
         split<D>(t, d);
-        mul(d, rhs, lane, o);
-    };
-    auto rhs_of = [&](uint32_t *rhs, const longlong2 *S, int mode) {
-        Tile<D> t;
-        Digits<D> d;
-        ld_priv<D>(S, lane, t);
-        split<D>(t, d);
-        put_rhs<D>(rhs, lane, d, mode);
-    };
-    auto add_to = [&](Tile<D> &a, const Tile<D> &b) {
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            a.re[e] += b.re[e];
-            a.im[e] += b.im[e];
-        }
     };
     // x / k!
     auto over = [&](i64 x, int k) -> i64 { return k <= 1 ? x : (k == 2 ? halve(x) : mulc(x, c_inv[k])); };
@@ -465,7 +449,8 @@ __global__ void __launch_bounds__(AdjCfg<D>::W * 32, 1) fx_adjoint_kernel(const 
 
         for (int rr = nr - 1; rr >= 0; --rr) {
             const int code = cls[rr], q = cls_q(code), rh = cls_r(code), s = cls_s(code);
-            Tile<D> T, M, o;
+            Tile<D> T, M;
+            Digits<D> dt, dm;  // digits of the T and M chains: each matrix is split once per use as both operands
             {
                 const longlong2 *src = reinterpret_cast<const longlong2 *>(gbuf + (size_t)rr * DD) + lane;
 #pragma unroll
@@ -490,39 +475,41 @@ __global__ void __launch_bounds__(AdjCfg<D>::W * 32, 1) fx_adjoint_kernel(const 
             st_priv<D>(SY, lane, T);
 
             // (P_j W_j)^T = W^T P^T, scaled by 2^-s like Y
-            rhs_of(r1, SP, kTrans);
-            mul_by(SW, r1, M);
+            split_of(SP, dt);
+            put_rhs<D>(r3, lane, dt, kTrans);
+            split_of(SW, dt);
+            mul(dt, r3, lane, M);
+            if (s > 0) {
 #pragma unroll
-            for (int e = 0; e < NE; ++e) {
-                M.re[e] = s > 0 ? (M.re[e] + (1ll << (s - 1))) >> s : M.re[e];
-                M.im[e] = s > 0 ? (M.im[e] + (1ll << (s - 1))) >> s : M.im[e];
+                for (int e = 0; e < NE; ++e) {
+                    M.re[e] = (M.re[e] + (1ll << (s - 1))) >> s;
+                    M.im[e] = (M.im[e] + (1ll << (s - 1))) >> s;
+                }
             }
             st_priv<D>(SD1, lane, M);  // D1
 
             // powers Y^k and their derivatives D_k; T = Y^q and M = D_q at the end
             uint32_t *rY = r1, *rD = r2;
-            rhs_of(rY, SY, kAntiHerm);
-            rhs_of(rD, SD1, kTrans);
-            if (q >= 2) {
-                mul_by(SY, rY, T);  // Y^2
-                mul_by(SD1, rY, M);
-                mul_by(SY, rD, o);
-                add_to(M, o);       // D2 = D1 Y + Y D1
-                if (q >= 3) {
+            split<D>(T, dt);
+            split<D>(M, dm);
+            put_rhs<D>(rY, lane, dt, kAntiHerm);
+            put_rhs<D>(rD, lane, dm, kTrans);
+            for (int k = 2; k <= q; ++k) {
+                // D2 = D1 Y + Y D1, D3 = D2 Y + Y^2 D1
+                mul_sum(dm, rY, dt, rD, lane, M);
+                mul(dt, rY, lane, T);
+                if (k < q) {
                     st_priv<D>(SY2, lane, T);
                     st_priv<D>(SD2, lane, M);
-                    mul_by(SY2, rY, T);  // Y^3
-                    mul_by(SD2, rY, M);
-                    mul_by(SY2, rD, o);
-                    add_to(M, o);        // D3 = D2 Y + Y^2 D1
+                    split<D>(T, dt);
+                    split<D>(M, dm);
                 }
             }
             if (rh > 1) {  // Y^q and D_q as right operands of the Horner steps
-                Digits<D> d;
-                split<D>(T, d);
-                put_rhs<D>(rY, lane, d, q == 2 ? kHerm : kAntiHerm);
-                split<D>(M, d);
-                put_rhs<D>(rD, lane, d, kTrans);
+                split<D>(T, dt);
+                put_rhs<D>(rY, lane, dt, q == 2 ? kHerm : kAntiHerm);
+                split<D>(M, dm);
+                put_rhs<D>(rD, lane, dm, kTrans);
             }
             auto add_block = [&](int b) {
                 const i64 a0 = c_inv_fx[q * b];
@@ -541,35 +528,30 @@ __global__ void __launch_bounds__(AdjCfg<D>::W * 32, 1) fx_adjoint_kernel(const 
             scale(T, q * rh);
             scale(M, q * rh);
             add_block(rh - 1);
-            for (int b = rh - 2; b >= 0; --b) {  // T <- T Y^q + B_b, M <- M Y^q + T D_q + its derivative
-                st_priv<D>(ST, lane, T);
-                st_priv<D>(SM, lane, M);
-                mul_by(SM, rY, M);
-                mul_by(ST, rD, o);
-                add_to(M, o);
-                mul_by(ST, rY, T);
-                add_block(b);
-            }
-            for (int i = 0; i < s; ++i) {  // M <- M T + T M, T <- T T
-                st_priv<D>(ST, lane, T);
-                st_priv<D>(SM, lane, M);
-                rhs_of(r1, ST, kTrans);
-                rhs_of(r2, SM, kTrans);
-                mul_by(SM, r1, M);
-                mul_by(ST, r2, o);
-                add_to(M, o);
-                mul_by(ST, r1, T);
+            // Horner steps T <- T Y^q + B_b, M <- M Y^q + T D_q + its derivative, then squarings M <- M T + T M, T <- T T
+            for (int i = rh - 2; i >= -s; --i) {
+                split<D>(T, dt);
+                split<D>(M, dm);
+                if (i < 0) {
+                    put_rhs<D>(rY, lane, dt, kTrans);
+                    put_rhs<D>(rD, lane, dm, kTrans);
+                }
+                mul_sum(dm, rY, dt, rD, lane, M);
+                mul(dt, rY, lane, T);
+                if (i >= 0) add_block(i);
             }
             // V = exp(Y) = U^T: M^T <- M'^T V^dagger, P^T <- P^T V^dagger, W^T <- V W^T
-            st_priv<D>(ST, lane, T);
-            st_priv<D>(SM, lane, M);
-            rhs_of(r1, ST, kHerm);  // the digits of conj(V) = (V^dagger)^T
-            rhs_of(r3, SW, kTrans);
-            mul_by(SM, r1, M);
-            mul_by(SP, r1, o);
-            st_priv<D>(SP, lane, o);
-            mul_by(ST, r3, o);
-            st_priv<D>(SW, lane, o);
+            split<D>(T, dt);
+            put_rhs<D>(r1, lane, dt, kHerm);  // the digits of conj(V) = (V^dagger)^T
+            split<D>(M, dm);
+            mul(dm, r1, lane, M);
+            split_of(SP, dm);
+            mul(dm, r1, lane, T);
+            st_priv<D>(SP, lane, T);
+            split_of(SW, dm);
+            put_rhs<D>(r3, lane, dm, kTrans);
+            mul(dt, r3, lane, T);
+            st_priv<D>(SW, lane, T);
             // M^T of the slice for the traces
 #pragma unroll
             for (int e = 0; e < NE; e += 2) {
