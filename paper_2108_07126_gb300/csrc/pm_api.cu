@@ -84,8 +84,10 @@ namespace {
 constexpr int kMaxDim = 256;
 constexpr int kMaxBatchDim = 128;  // the batched kernel's block-level bodies go up to D = 128
 constexpr int kMaxSmallDim = 16;  // larger dimensions use one thread block per leaf
-constexpr int kLeafMinSteps = 8;    // fewer blocks for short runs: each leaf gets >= 8 slices (FP32)
-constexpr int kLeafMinSteps64 = 2;  // the same for FP64, whose slices cost far more than the tree
+// Fewer blocks for short runs: each leaf gets at least two slices.  A slice is a chain of dependent products, dearer than
+// a level of the tree (FP32, 8 -> 2 slices: d = 16, N = 2048 158 -> 94 us, gradient d = 8, N = 1501 600 -> 261 us).
+constexpr int kLeafMinSteps = 2;    // FP32
+constexpr int kLeafMinSteps64 = 2;  // FP64
 
 struct Workspace {
     void *ptr = nullptr;
