@@ -372,8 +372,9 @@ __global__ void __launch_bounds__(AdjCfg<D>::W * 32, 1) fx_adjoint_kernel(const 
 
     unsigned flags = 0, bad = 0;
     const double gscale = -2.0 / p.d_true;  // 1 / d is in W
-    const double vn = p.z[3];
-    const int ve = (vn > 1.5 && vn < 1e300) ? ilogb(vn) / 2 + 1 : 0;
+    // W = conj(z) / d V^dagger S enters scaled by a power of two to a norm near one (p.z[3] >= ||V||_2^2)
+    const double wn = sqrt(p.z[3] * (p.z[0] * p.z[0] + p.z[1] * p.z[1])) / p.d_true;
+    const int ve = (wn > 1e-150 && wn < 1e150) ? ilogb(wn) + 1 : 0;
 
     auto split_of = [&](const longlong2 *S, Digits<D> &d) {
         Tile<D> t;

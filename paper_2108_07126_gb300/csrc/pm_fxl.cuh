@@ -41,7 +41,7 @@ __device__ __forceinline__ i64 to_fixed(double v, bool &bad) {
     bad = bad || e >= 1024;
     const u64 m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
     const int sh = e - 1075 + fx::F;  // <= 4 for |v| < 2
-    const u64 q = sh >= 0 ? m << (sh & 7) : (sh > -60 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0ull);
+    const u64 q = sh >= 0 ? m << (sh & 7) : (sh > -60 ? fx::round_even(m, -sh) : 0ull);
     return (i64)b < 0 ? -(i64)q : (i64)q;
 }
 

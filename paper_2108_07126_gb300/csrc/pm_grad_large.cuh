@@ -164,9 +164,9 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
     const int len = (int)(N * (leaf + 1) / L - j0);
     if (len <= 0) return;  // uniform over the block
     const Real zr = (Real)p.z[0], zi = (Real)p.z[1];
-    // V enters scaled by a power of two to a spectral norm of about one at most (p.z[3] >= ||V||_2^2)
+    // V enters scaled by a power of two to a spectral norm of about one (p.z[3] >= ||V||_2^2)
     const double vn = p.z[3];
-    const int ve = (vn > 1.5 && vn < 1e300) ? ilogb(vn) / 2 + 1 : 0;
+    const int ve = ((vn > 1.5 || vn < 0.5) && vn > 1e-200 && vn < 1e200) ? (int)floor(0.5 * log2(vn)) + 1 : 0;
     const Real vback = (Real)ldexp(1.0, ve), vscale = (Real)ldexp(1.0, -ve);
     const Real gscale = (Real)(-2.0 / (p.d_true * p.d_true)) * vback;
     unsigned flags = 0;
