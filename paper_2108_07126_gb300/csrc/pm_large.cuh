@@ -15,6 +15,7 @@
 
 #include "pm_fused.cuh"
 #include "pm_fxl.cuh"
+#include "pm_fxu.cuh"
 #include "pm_tc_small.cuh"
 #include "pm_umma.cuh"
 
@@ -50,7 +51,7 @@ template <typename Real, int D> struct LGeo {
 };
 
 // TCM: 0 = CUDA-core products, 2 = 3xTF32 with tcgen05 (D = 128, 256: 128 x 128 output blocks),
-// 3 = split BF16x3 with tcgen05 (D = 128, 256), 4 / 5 = 3xTF32 / split BF16x3 with tcgen05 in the
+// 3 = split BF16x3 with tcgen05 (D = 128, 256), 6 = FP64 digit products with tcgen05 (D >= 64; FP64 with 0: mma.sync), 4 / 5 = 3xTF32 / split BF16x3 with tcgen05 in the
 // shared-memory body of pm_tc_small.cuh (D = 32, 64)
 template <int TCM> __host__ __device__ constexpr int tcm_format() { return (TCM == 3 || TCM == 5) ? umma::kBF16x3 : umma::kTF32x3; }
 
@@ -64,7 +65,12 @@ __host__ __device__ inline size_t large_panel_bytes() {
     size_t b = LGeo<Real, D>::PANEL_BYTES;
     if (LGeo<double, D>::PANEL_BYTES > b) b = LGeo<double, D>::PANEL_BYTES;
     if ((std::is_same<Real, double>::value || tree_on_digits<D>()) && fxl::mm_bytes<D>() > b) b = fxl::mm_bytes<D>();
-    if (TCM >= 2 && umma::kSmemBytes > b) b = umma::kSmemBytes;
+    if (std::is_same<Real, double>::value && D >= 64) {  // the tcgen05 panels, or the padded packed exponent in their place
+        if (fxu::BYTES > b) b = fxu::BYTES;
+        if (D <= 128 && (size_t)D * (D + 1) * sizeof(double) > b) b = (size_t)D * (D + 1) * sizeof(double);
+    } else if (TCM >= 2 && umma::kSmemBytes > b) {
+        b = umma::kSmemBytes;
+    }
     return b;
 }
 
@@ -85,7 +91,7 @@ __host__ __device__ inline size_t large_front_bytes() {
 
 template <typename Real, int D, int TCM = 0>
 __host__ __device__ inline size_t large_smem_bytes(int n_basis) {
-    if constexpr (TCM >= 4) {
+    if constexpr (TCM == 4 || TCM == 5) {
         // the tensor-core body, and the FP64 / FP32 panels of the arrival tree that may follow it
         size_t b = tcs::smem_bytes<D, tcm_format<TCM>()>(n_basis);
         if (fxl::mm_bytes<D>() > b) b = fxl::mm_bytes<D>();
@@ -245,6 +251,7 @@ __device__ __forceinline__ void large_mm(const typename Cx<Real>::T *A, const ty
     } else if constexpr (std::is_same<Real, double>::value) {
         // digit products; the Clenshaw recurrence of the Chebyshev series leaves their range (|entry| < 2)
         if (cheb) cta_mm<Real, D>(A, B, Cout, panels);
+        else if constexpr (TCM == 6) fxu::cta_mm<D>(A, B, Cout, panels, d, *uc);
         else fxl::cta_mm<D>(A, B, Cout, panels, d);
     } else {
         cta_mm<Real, D>(A, B, Cout, panels);
@@ -299,6 +306,11 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
     const bool cheb = p.cheb_m != nullptr;
     const int mch = cheb ? *p.cheb_m : 0;
     const Real ib = cheb ? (Real)*p.cheb_inv_beta : Real(0);
+    // FP64: the digit products use the leading ext rows and columns only, and so do the element passes (on the FP64
+    // pipe they would cost as much as the products); at() maps a dense index over ext x ext to the frame
+    constexpr bool kExt = std::is_same<Real, double>::value;
+    const int ext = (kExt && !cheb) ? (D == 32 ? 32 : fxl::extent(p.d_out)) : D, n_el = ext * ext;
+    auto at = [&](int e) { return kExt ? (e / ext) * D + e % ext : e; };
 
     for (int t = 0; t < len; ++t) {
         const int64_t j = j0 + t;
@@ -316,6 +328,22 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
         // memory for the resident bodies, in the global scratch otherwise)
         Real *gpk = (TCM >= 2 && D <= 128) ? (Real *)panels : (Real *)P0;
 
+        if constexpr (kExt) {
+            for (int e4 = tid; e4 < n_el / 4; e4 += kLargeThreads) {
+                const int i = (4 * e4) / ext, jj = (4 * e4) % ext;
+                Real v[4] = {Real(0), Real(0), Real(0), Real(0)};
+#pragma unroll 4
+                for (int b = 0; b < nb; ++b) {
+                    const Real g = gam[b];
+                    Real w[4];
+                    ld4<Real>(packed + (size_t)b * DD + i * D + jj, w);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[u] = fma(g, w[u], v[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) gpk[i * GLD + jj + u] = v[u];
+            }
+        } else
         // packed exponent sum_b gamma_b P_b: EP groups of four entries per thread and step, the
         // basis loop unrolled, so that 4 EP independent 16-byte loads from L2 are in flight (the
         // basis is read once per slice and does not fit in shared memory)
@@ -350,8 +378,8 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
         __syncthreads();
         // Hermitian unpack (upper triangle: Re, strict lower: Im) into A = -i G / 2^s, or into
         // X = G / beta for the Chebyshev series
-        for (int e = tid; e < DD; e += kLargeThreads) {
-            const int i = e / D, jj = e % D;
+        for (int l = tid; l < n_el; l += kLargeThreads) {
+            const int e = at(l), i = e / D, jj = e % D;
             const Real a = gpk[i * GLD + jj], b = gpk[jj * GLD + i];
             const Real re = (i <= jj) ? a : b;
             const Real im = (i > jj) ? a : ((i < jj) ? -b : Real(0));
@@ -412,18 +440,20 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             const Real a1 = (q >= 2) ? coef<Real>(p, q * b + 1) : Real(0);
             const Real a2 = (q >= 3) ? coef<Real>(p, q * b + 2) : Real(0);
             const bool scaled = scale != Real(1);
-            for (int e0 = tid; e0 < DD; e0 += 4 * kLargeThreads) {
+            for (int e0 = tid; e0 < n_el; e0 += 4 * kLargeThreads) {
                 C v[4], x1[4], x2[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int e = e0 + u * kLargeThreads;
+                    if (kExt && e0 + u * kLargeThreads >= n_el) break;
+                    const int e = at(e0 + u * kLargeThreads);
                     v[u] = src[e];
                     if (q >= 2) x1[u] = SX[e];
                     if (q >= 3) x2[u] = SX2[e];
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int e = e0 + u * kLargeThreads;
+                    if (kExt && e0 + u * kLargeThreads >= n_el) break;
+                    const int e = at(e0 + u * kLargeThreads);
                     C w = v[u];
                     if (scaled) w = Cx<Real>::make(v[u].x * scale, v[u].y * scale);
                     w.x += ((e / D) == (e % D)) ? a0 : Real(0);
@@ -554,13 +584,13 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
 // matrices in a global scratch region for D = 128, 256
 template <typename Real, int D, int TC>
 __host__ __device__ constexpr int large_tcm() {
-    return (TC == 0 || !std::is_same<Real, float>::value) ? 0 : (D <= 64 ? (TC == 2 ? 5 : 4) : (TC == 2 ? 3 : 2));
+    return std::is_same<Real, double>::value ? (D >= 64 ? 6 : 0) : TC == 0 ? 0 : (D <= 64 ? (TC == 2 ? 5 : 4) : (TC == 2 ? 3 : 2));
 }
 
 // blocks per SM the large kernel is compiled for: two for the tensor-core body at D = 32
 template <typename Real, int D, int TC>
 __host__ __device__ constexpr int large_min_blocks() {
-    return large_tcm<Real, D, TC>() >= 4 ? tcs::Cfg<D, tcm_format<large_tcm<Real, D, TC>()>()>::MIN_BLOCKS : 1;
+    return (large_tcm<Real, D, TC>() == 4 || large_tcm<Real, D, TC>() == 5) ? tcs::Cfg<D, tcm_format<large_tcm<Real, D, TC>()>()>::MIN_BLOCKS : 1;
 }
 
 template <typename Real, int D, int INTEG, int TC = 0>
@@ -570,7 +600,7 @@ __global__ void __launch_bounds__(kLargeThreads, large_min_blocks<Real, D, TC>()
     using C = typename Cx<Real>::T;
     constexpr int TCM = large_tcm<Real, D, TC>();
     C *ws = (C *)scratch + (size_t)blockIdx.x * kLargeSlots * D * D;
-    if constexpr (TCM >= 4) {
+    if constexpr (TCM == 4 || TCM == 5) {
         __shared__ __align__(8) uint64_t s_mbar[umma::kBars];
         __shared__ uint32_t s_tmem;
         __shared__ int s_abort;
