@@ -1405,7 +1405,7 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     const size_t cap = (size_t)ctx->opt_workspace_mb << 20;
     while (c_sub > 1 && (size_t)TG * c_sub * DD * csz > cap) c_sub = (c_sub + 1) / 2;
     const int64_t n_ckpt = std::max<int64_t>(1, (maxlen + c_sub - 1) / c_sub);
-    if (!fx_adjoint) {
+    if (!fx_adjoint && !(large && fp64)) {  // one sweep stores no prefixes
         if ((st = ws_reserve(ctx, ctx->gpbuf, (size_t)TG * c_sub * DD * csz))) return st;
         if ((st = ws_reserve(ctx, ctx->gckpt, (size_t)TG * n_ckpt * DD * csz))) return st;
     }

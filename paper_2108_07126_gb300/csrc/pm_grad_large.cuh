@@ -123,7 +123,8 @@ __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(siz
 template <typename Real, int D> struct AdjLayout {
     using C = typename Cx<Real>::T;
     // after the product's panels
-    static constexpr size_t GAM = std::is_same<Real, double>::value ? fxl::mm_bytes<D>() : LGeo<Real, D>::PANEL_BYTES;
+    static constexpr size_t GAM = std::is_same<Real, double>::value ? (D >= 64 ? fxu::BYTES : fxl::mm_bytes<D>())
+                                                                    : LGeo<Real, D>::PANEL_BYTES;
     static constexpr size_t TRC = GAM + align16(kMaxBasis * sizeof(Real));    // Tr(M B_e)
     static constexpr size_t RED = TRC + align16(kMaxBasis * sizeof(C));       // per-warp partial traces
     static constexpr size_t BYTES = RED + align16((size_t)kMaxBasis * 8 * sizeof(C));
@@ -132,13 +133,16 @@ template <typename Real, int D> struct AdjLayout {
 template <typename Real, int D>
 __host__ __device__ constexpr size_t adjoint_large_smem_bytes() { return AdjLayout<Real, D>::BYTES; }
 
-// One block per leaf (grid = p.n_leaves); scratch: kGradSlots D x D complex matrices per block.
+// The sweeps of one leaf by one block (leaf = blockIdx.x); scratch: kGradSlots D x D complex matrices per block.  FP64 runs
+// one backward sweep: with the prefix after the slice in place of the one before it (pm_fx_grad.cuh),
+// M = U^dagger M' and P_{j-1} = U^dagger P_j follow from the exponential the derivative needs anyway -- 19 products a
+// slice instead of 23, no stored prefixes.  FP32 keeps the two sweeps (the inverse of a rounded U drifts there).
 template <typename Real, int D, int INTEG>
-__global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams p, void *scratch) {
+__device__ __forceinline__ void adjoint_large_body(const GradParams &p, void *scratch, unsigned char *smem, umma::Ctx *uc) {
+    constexpr bool kUmma = std::is_same<Real, double>::value && D >= 64;  // products on tcgen05
     using C = typename Cx<Real>::T;
     using AL = AdjLayout<Real, D>;
     constexpr int DD = D * D, NT = 256;
-    extern __shared__ __align__(16) unsigned char smem[];
     unsigned char *panels = smem;
     Real *gam = (Real *)(smem + AL::GAM);
     C *Ttr = (C *)(smem + AL::TRC);
@@ -172,7 +176,8 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
     unsigned flags = 0;
 
     auto mm = [&](const C *A, const C *B, C *Cm) {  // ends with a barrier
-        if constexpr (std::is_same<Real, double>::value) fxl::cta_mm<D>(A, B, Cm, panels, (int)p.d_true);
+        if constexpr (kUmma) fxu::cta_mm<D>(A, B, Cm, panels, (int)p.d_true, *uc);
+        else if constexpr (std::is_same<Real, double>::value) fxl::cta_mm<D>(A, B, Cm, panels, (int)p.d_true);
         else cta_mm<Real, D>(A, B, Cm, panels);
     };
     auto ld_glob = [&](C *S, const double2 *src) {
@@ -324,7 +329,8 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
         TL = t;
     };
 
-    const int c_sub = p.c_sub;
+    constexpr bool kOne = std::is_same<Real, double>::value;  // one sweep
+    const int c_sub = kOne ? len : p.c_sub;
     const int nsub = (len + c_sub - 1) / c_sub;
     // checkpoint pass: prefixes at the start of every sub-chunk
     if (nsub > 1) {
@@ -344,9 +350,9 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
         const int a = sub * c_sub;
         const int nt = min(c_sub, len - a);
         if (nsub > 1) copy(P, ckpt + (size_t)sub * DD);
-        else ld_glob(P, p.pin + (size_t)leaf * DD);
+        else ld_glob(P, p.pin + (size_t)(leaf + kOne) * DD);  // one sweep: the prefix at the leaf's end
         // forward sweep over the sub-chunk: store P_{j-1}, advance
-        for (int t = 0; t < nt; ++t) {
+        for (int t = 0; !kOne && t < nt; ++t) {
             copy(pbuf + (size_t)t * DD, P);
             block_exp(prep(j0 + a + t, false), false);
             advance_prefix();
@@ -354,9 +360,9 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
         // backward sweep
         for (int t = nt - 1; t >= 0; --t) {
             const int64_t j = j0 + a + t;
-            copy(P, pbuf + (size_t)t * DD);
+            if (!kOne) copy(P, pbuf + (size_t)t * DD);
             const int code = prep(j, true);
-            // Lambda = P_{j-1} W, scaled like A
+            // Lambda = P_{j-1} W (one sweep: P_j W), scaled like A
             mm(P, W, D1);
             {
                 const Real sc = pow2neg<Real>(cls_s(code));
@@ -364,6 +370,21 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
                 __syncthreads();
             }
             block_exp(code, true);
+            if (kOne) {  // M = U^dagger M', P_{j-1} = U^dagger P_j
+                for (int e = tid; e < DD; e += NT) {
+                    const C v = U[e];
+                    T3[(e % D) * D + e / D] = Cx<Real>::make(v.x, -v.y);
+                }
+                __syncthreads();
+                mm(T3, M, TR);
+                mm(T3, P, TL);
+                C *x = M;
+                M = TR;
+                TR = x;
+                x = P;
+                P = TL;
+                TL = x;
+            }
             // T_e = Tr(M B_e) for every kept basis matrix from its packed real form (upper
             // triangle: Re, strict lower: Im); element (i, jj) of M meets B_e[jj][i]
             for (int e = 0; e < nb; ++e) {
@@ -454,6 +475,22 @@ __global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams 
         }
     }
     if (flags) atomicOr(p.status, flags);
+}
+
+template <typename Real, int D, int INTEG>
+__global__ void __launch_bounds__(256, 1) adjoint_large_kernel(const GradParams p, void *scratch) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    if constexpr (std::is_same<Real, double>::value && D >= 64) {
+        __shared__ __align__(8) uint64_t s_mbar[umma::kBars];
+        __shared__ uint32_t s_tmem;
+        __shared__ int s_abort;
+        umma::Ctx cx;
+        umma::setup(cx, s_mbar, &s_tmem, &s_abort, p.status);
+        adjoint_large_body<Real, D, INTEG>(p, scratch, smem, &cx);
+        umma::teardown(cx);
+    } else {
+        adjoint_large_body<Real, D, INTEG>(p, scratch, smem, nullptr);
+    }
 }
 
 template <typename Real, int INTEG, int D>
