@@ -84,10 +84,12 @@ namespace {
 constexpr int kMaxDim = 256;
 constexpr int kMaxBatchDim = 128;  // the batched kernel's block-level bodies go up to D = 128
 constexpr int kMaxSmallDim = 16;  // larger dimensions use one thread block per leaf
-// Fewer blocks for short runs: each leaf gets at least two slices.  A slice is a chain of dependent products, dearer than
-// a level of the tree (FP32, 8 -> 2 slices: d = 16, N = 2048 158 -> 94 us, gradient d = 8, N = 1501 600 -> 261 us).
-constexpr int kLeafMinSteps = 2;    // FP32
-constexpr int kLeafMinSteps64 = 2;  // FP64
+constexpr int kLeafMinSteps = 2;    // fewer blocks for short runs: each leaf gets >= 2 slices (FP32)
+// FP32 gradients of d = 5..8 up to this length run in FP64 and round the result: a short run is bound by latency, and the
+// one-sweep FP64 adjoint has less of it (d = 8, FP32 / FP64 path: N = 64 200 / 175 us, 1024 256 / 203 us, 1501 249 / 207 us,
+// 3000 261 / 269 us; d = 9..16 is slower at every length, N = 64 251 / 450 us).
+constexpr int64_t kGradVia64Steps = 2048;
+constexpr int kLeafMinSteps64 = 2;  // the same for FP64, whose slices cost far more than the tree
 
 struct Workspace {
     void *ptr = nullptr;
@@ -1311,12 +1313,13 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     if (prec != PARAMENT_PREC_FP64 && prec != PARAMENT_PREC_FP32)
         return set_err(ctx, PARAMENT_ERR_UNSUPPORTED, "gradient precision must be FP64 or FP32");
     DeviceGuard guard(ctx->device);
-    const int fp64 = prec == PARAMENT_PREC_FP64;
     const int Dp = ctx->dpad, d = ctx->dim, K = ctx->K;
+    const int64_t N = ctx->n_steps;
+    const bool via64 = prec == PARAMENT_PREC_FP32 && Dp == 8 && N <= kGradVia64Steps;
+    const int fp64 = prec == PARAMENT_PREC_FP64 || via64;
     const size_t DD = (size_t)Dp * Dp;
     const size_t esz = ctx->dtype == PARAMENT_C128 ? 16 : 8;
-    const size_t rsz = fp64 ? 8 : 4;
-    const int64_t N = ctx->n_steps;
+    const size_t rsz = fp64 ? 8 : 4;  // of the arithmetic; grad_out is float with FP32
     int st;
 
     // V (host or device) -> V^dagger padded, FP64
@@ -1413,9 +1416,9 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
 
     void *gdst = grad_out;
     const bool host_g = !is_device_ptr(grad_out);
-    const size_t gbytes = (size_t)K * ctx->S * rsz;
-    if (host_g) {
-        if ((st = ws_reserve(ctx, ctx->ggrad, std::max<size_t>(gbytes, 8)))) return st;
+    const size_t gcount = (size_t)K * ctx->S, gbytes = gcount * rsz;
+    if (host_g || via64) {  // via64: the double gradient, then (host) the float one
+        if ((st = ws_reserve(ctx, ctx->ggrad, std::max<size_t>(gbytes + (via64 && host_g ? gcount * 4 : 0), 8)))) return st;
         gdst = ctx->ggrad.ptr;
     }
 
@@ -1488,7 +1491,16 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     }
     ctx->last.grad_subchunk = (int32_t)c_sub;
 
-    if (host_g && gbytes) PM_CUDA(cudaMemcpyAsync(grad_out, gdst, gbytes, cudaMemcpyDeviceToHost, ctx->stream));
+    size_t out_bytes = gbytes;
+    if (via64 && gcount) {
+        float *gf = host_g ? (float *)((double *)gdst + gcount) : (float *)grad_out;
+        convert_kernel<double, float><<<(int)std::min<size_t>((gcount + 255) / 256, 4096), 256, 0, ctx->stream>>>(
+            (const double *)gdst, gf, (int64_t)gcount);
+        PM_CUDA(cudaGetLastError());
+        gdst = gf;
+        out_bytes = gcount * 4;
+    }
+    if (host_g && gbytes) PM_CUDA(cudaMemcpyAsync(grad_out, gdst, out_bytes, cudaMemcpyDeviceToHost, ctx->stream));
     if (host_u) PM_CUDA(cudaMemcpyAsync(U_out, udst, (size_t)d * d * esz, cudaMemcpyDeviceToHost, ctx->stream));
     if (loss_out) {
         double z[4];
