@@ -337,6 +337,8 @@ class Propagator:
 
         self._torch = torch
         self.device = torch.device("cuda", device)
+        # the raw handle of the current stream without building a Stream object (1.5 us of a 25 us call)
+        self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
         self.ctx = parament_create(device, torch.cuda.current_stream(self.device).cuda_stream)
         self._keep = []
         self.dim = None
@@ -354,7 +356,11 @@ class Propagator:
             pass
 
     def _sync_stream(self):
-        parament_set_stream(self.ctx, self._torch.cuda.current_stream(self.device).cuda_stream)
+        raw = self._raw_stream
+        st = _lib.parament_set_stream(self.ctx, (raw(self.device.index) if raw is not None
+                                                 else self._torch.cuda.current_stream(self.device).cuda_stream) or None)
+        if st:
+            _check(st, self.ctx)
 
     def set_option(self, key: int, value: int):
         parament_set_option(self.ctx, key, value)
@@ -387,22 +393,29 @@ class Propagator:
         c = torch.as_tensor(c)
         if c.dtype not in (torch.float32, torch.float64):
             c = c.to(torch.float64)
-        c = c.to(self.device).contiguous()
+        if c.device != self.device or not c.is_contiguous():
+            c = c.to(self.device).contiguous()
+        n = c.numel()
         if n_steps is None:
-            S = c.shape[-1] if c.numel() else 0
+            S = c.shape[-1] if n else 0
             n_steps = {"midpoint": S, "magnus4_gl2": S // 2, "magnus4_simpson": max(S - 1, 0) // 2}[self.integrator]
         self._sync_stream()
-        parament_set_controls(self.ctx, c.data_ptr() if c.numel() else None,
-                              PARAMENT_F64 if c.dtype == torch.float64 else PARAMENT_F32, n_steps, dt)
+        # the library directly (a short call's time is host time)
+        st = _lib.parament_set_controls(self.ctx, c.data_ptr() if n else None,
+                                        PARAMENT_F64 if c.dtype == torch.float64 else PARAMENT_F32, int(n_steps), float(dt))
+        if st:
+            _check(st, self.ctx)
         self._ctrl = c
         self.n_steps = n_steps
 
     def propagate(self, prec: str = "fp64", out=None):
         torch = self._torch
         if out is None:
-            out = torch.empty(self.dim, self.dim, dtype=self.dtype, device=self.device)
+            out = torch.empty((self.dim, self.dim), dtype=self.dtype, device=self.device)
         self._sync_stream()
-        parament_propagate(self.ctx, out.data_ptr(), PRECISIONS[prec])
+        st = _lib.parament_propagate(self.ctx, out.data_ptr(), PRECISIONS[prec])
+        if st:
+            _check(st, self.ctx)
         return out
 
     def propagate_trajectory(self, prec: str = "fp64", every: int = 1, psi0=None, out=None):
