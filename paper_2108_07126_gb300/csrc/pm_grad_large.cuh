@@ -176,7 +176,7 @@ __device__ __forceinline__ void adjoint_large_body(const GradParams &p, void *sc
     unsigned flags = 0;
 
     auto mm = [&](const C *A, const C *B, C *Cm) {  // ends with a barrier
-        if constexpr (kUmma) fxu::cta_mm<D>(A, B, Cm, panels, (int)p.d_true, *uc);
+        if constexpr (kUmma) fxu::cta_mm<D, 256, double2>(A, B, Cm, panels, (int)p.d_true, *uc);
         else if constexpr (std::is_same<Real, double>::value) fxl::cta_mm<D>(A, B, Cm, panels, (int)p.d_true);
         else cta_mm<Real, D>(A, B, Cm, panels);
     };

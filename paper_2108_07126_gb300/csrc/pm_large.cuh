@@ -251,7 +251,6 @@ __device__ __forceinline__ void large_mm(const typename Cx<Real>::T *A, const ty
     } else if constexpr (std::is_same<Real, double>::value) {
         // digit products; the Clenshaw recurrence of the Chebyshev series leaves their range (|entry| < 2)
         if (cheb) cta_mm<Real, D>(A, B, Cout, panels);
-        else if constexpr (TCM == 6) fxu::cta_mm<D>(A, B, Cout, panels, d, *uc);
         else fxl::cta_mm<D>(A, B, Cout, panels, d);
     } else {
         cta_mm<Real, D>(A, B, Cout, panels);
@@ -282,6 +281,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
     // when the tensor-core stages leave room, else in a free scratch slot
     constexpr bool kGpkShared = (TCM >= 2 && D <= 128) || kResident;  // D = 256: 263 KB, too large
     static_assert(DD % (4 * kLargeThreads) == 0, "element passes take four elements per thread and step");
+    constexpr int nt = kLargeThreads;
     constexpr int GLD = kGpkShared ? D + 1 : D;
     const Real *packed = (const Real *)p.packed;
 
@@ -290,7 +290,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
 
     // R = I, or in trajectory mode the product of every slice before the leaf (FP64 prefix)
     const bool traj = p.traj_out != nullptr;
-    for (int e = tid; e < DD; e += kLargeThreads) {
+    for (int e = tid; e < DD; e += nt) {
         if (traj) {
             const double2 v = p.traj_pin[(size_t)blk * DD + e];
             SR[e] = Cx<Real>::make((Real)v.x, (Real)v.y);
@@ -307,10 +307,9 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
     const int mch = cheb ? *p.cheb_m : 0;
     const Real ib = cheb ? (Real)*p.cheb_inv_beta : Real(0);
     // FP64: the digit products use the leading ext rows and columns only, and so do the element passes (on the FP64
-    // pipe they would cost as much as the products); at() maps a dense index over ext x ext to the frame
+    // pipe they would cost as much as the products)
     constexpr bool kExt = std::is_same<Real, double>::value;
     const int ext = (kExt && !cheb) ? (D == 32 ? 32 : fxl::extent(p.d_out)) : D, n_el = ext * ext;
-    auto at = [&](int e) { return kExt ? (e / ext) * D + e % ext : e; };
 
     for (int t = 0; t < len; ++t) {
         const int64_t j = j0 + t;
@@ -329,7 +328,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
         Real *gpk = (TCM >= 2 && D <= 128) ? (Real *)panels : (Real *)P0;
 
         if constexpr (kExt) {
-            for (int e4 = tid; e4 < n_el / 4; e4 += kLargeThreads) {
+            for (int e4 = tid; e4 < n_el / 4; e4 += nt) {
                 const int i = (4 * e4) / ext, jj = (4 * e4) % ext;
                 Real v[4] = {Real(0), Real(0), Real(0), Real(0)};
 #pragma unroll 4
@@ -378,19 +377,25 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
         __syncthreads();
         // Hermitian unpack (upper triangle: Re, strict lower: Im) into A = -i G / 2^s, or into
         // X = G / beta for the Chebyshev series
-        for (int l = tid; l < n_el; l += kLargeThreads) {
-            const int e = at(l), i = e / D, jj = e % D;
+        auto unpack = [&](int i, int jj) {
+            const int e = i * D + jj;
             const Real a = gpk[i * GLD + jj], b = gpk[jj * GLD + i];
             const Real re = (i <= jj) ? a : b;
             const Real im = (i > jj) ? a : ((i < jj) ? -b : Real(0));
             SX[e] = cheb ? Cx<Real>::make(re * ib, im * ib) : Cx<Real>::make(im * sc, -re * sc);
+        };
+        if constexpr (kExt) {
+            for (int i = tid >> 4; i < ext; i += nt >> 4)
+                for (int jj = tid & 15; jj < ext; jj += 16) unpack(i, jj);
+        } else {
+            for (int e = tid; e < DD; e += nt) unpack(e / D, e % D);
         }
         __syncthreads();
         if (cheb) {
             // Clenshaw: D_m = a_m I, D_{m+1} = 0; D_k = a_k I + 2 X D_{k+1} - D_{k+2}; U = D_0 - D_2
             const C *ak = (const C *)p.cheb_coef;
             C *d1 = SX2, *d2 = SX3, *nw = P0;
-            for (int e = tid; e < DD; e += kLargeThreads) {
+            for (int e = tid; e < DD; e += nt) {
                 const bool diag = (e / D) == (e % D);
                 d1[e] = diag ? ak[mch] : Cx<Real>::make(Real(0), Real(0));
                 d2[e] = Cx<Real>::make(Real(0), Real(0));
@@ -399,7 +404,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             for (int k = mch - 1; k >= 0; --k) {
                 large_mm<Real, D, TCM>(SX, d1, nw, panels, uc, p.d_out, true);
                 const C a_k = ak[k];
-                for (int e = tid; e < DD; e += kLargeThreads) {
+                for (int e = tid; e < DD; e += nt) {
                     const C x = nw[e], y = d2[e];
                     C v = Cx<Real>::make(Real(2) * x.x - y.x, Real(2) * x.y - y.y);
                     if ((e / D) == (e % D)) {
@@ -440,20 +445,20 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             const Real a1 = (q >= 2) ? coef<Real>(p, q * b + 1) : Real(0);
             const Real a2 = (q >= 3) ? coef<Real>(p, q * b + 2) : Real(0);
             const bool scaled = scale != Real(1);
-            for (int e0 = tid; e0 < n_el; e0 += 4 * kLargeThreads) {
+            auto four = [&](int e0, int stride, int n) {  // elements e0, e0 + stride, ... (n of them, at most four)
                 C v[4], x1[4], x2[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    if (kExt && e0 + u * kLargeThreads >= n_el) break;
-                    const int e = at(e0 + u * kLargeThreads);
+                    if (kExt && u >= n) break;
+                    const int e = e0 + u * stride;
                     v[u] = src[e];
                     if (q >= 2) x1[u] = SX[e];
                     if (q >= 3) x2[u] = SX2[e];
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    if (kExt && e0 + u * kLargeThreads >= n_el) break;
-                    const int e = at(e0 + u * kLargeThreads);
+                    if (kExt && u >= n) break;
+                    const int e = e0 + u * stride;
                     C w = v[u];
                     if (scaled) w = Cx<Real>::make(v[u].x * scale, v[u].y * scale);
                     w.x += ((e / D) == (e % D)) ? a0 : Real(0);
@@ -467,6 +472,12 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
                     }
                     T[e] = w;
                 }
+            };
+            if constexpr (kExt) {  // rows of 16 threads: no divisions by ext
+                for (int i = tid >> 4; i < ext; i += nt >> 4)
+                    for (int jj = tid & 15; jj < ext; jj += 64) four(i * D + jj, 16, (ext - jj + 15) >> 4);
+            } else {
+                for (int e0 = tid; e0 < DD; e0 += 4 * nt) four(e0, nt, 4);
             }
             __syncthreads();
         };
@@ -495,14 +506,14 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             const int64_t o = j / p.traj_every;
             const int d = p.d_out;
             if (p.traj_psi0 == nullptr) {
-                for (int e = tid; e < d * d; e += kLargeThreads) {
+                for (int e = tid; e < d * d; e += nt) {
                     const C v = SR[(e / d) * D + e % d];
                     const size_t at = (size_t)o * d * d + e;
                     if (p.out_c128) ((double2 *)p.traj_out)[at] = make_double2((double)v.x, (double)v.y);
                     else ((float2 *)p.traj_out)[at] = make_float2((float)v.x, (float)v.y);
                 }
             } else {
-                for (int i = tid; i < d; i += kLargeThreads) {
+                for (int i = tid; i < d; i += nt) {
                     Real re = 0, im = 0;
                     for (int k = 0; k < d; ++k) {
                         const C a = SR[i * D + k];
@@ -534,19 +545,19 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
     // truncating accumulation of the tensor cores, drift R off the unitary group along a leaf)
     if constexpr (std::is_same<Real, float>::value) {
         if (p.unitary_step && len > 0) {
-            for (int e = tid; e < DD; e += kLargeThreads) {
+            for (int e = tid; e < DD; e += nt) {
                 const C v = SR[(e % D) * D + e / D];
                 P0[e] = Cx<Real>::make(v.x, -v.y);  // R^dagger
             }
             __syncthreads();
             large_mm<Real, D, TCM>(P0, SR, P1, panels, uc, p.d_out);  // R^dagger R
-            for (int e = tid; e < DD; e += kLargeThreads) {
+            for (int e = tid; e < DD; e += nt) {
                 const C v = P1[e];
                 P1[e] = Cx<Real>::make(((e / D) == (e % D) ? Real(3) : Real(0)) - v.x, -v.y);
             }
             __syncthreads();
             large_mm<Real, D, TCM>(SR, P1, P0, panels, uc, p.d_out);  // R (3 I - R^dagger R)
-            for (int e = tid; e < DD; e += kLargeThreads) {
+            for (int e = tid; e < DD; e += nt) {
                 const C v = P0[e];
                 SR[e] = Cx<Real>::make(Real(0.5) * v.x, Real(0.5) * v.y);
             }
@@ -565,7 +576,7 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
     // block partial (the leaf product) in FP64
     {
         double2 *dst = p.partials + (size_t)blk * DD;
-        for (int e = tid; e < DD; e += kLargeThreads) {
+        for (int e = tid; e < DD; e += nt) {
             C v = SR[e];
             // the digit products leave the padding beyond the dimension undefined: the identity there
             if (std::is_same<Real, double>::value && max(e / D, e % D) >= p.d_out)
@@ -574,6 +585,191 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
             if (p.leaf_out) p.leaf_out[(size_t)blk * DD + e] = dst[e];
             if (p.block_out) p.block_out[(size_t)blk * DD + e] = dst[e];
         }
+    }
+    __threadfence();
+    __syncthreads();
+}
+
+// FP64 slices of D >= 64: the work of large_body's Taylor branch with the working matrices as fixed-point numbers
+// x = q 2^-56 (every one is bounded, see pm_digits.cuh), so that the operands of the tcgen05 products are split without a
+// conversion and the Horner passes leave the FP64 pipe.  Sixteen warps: the splits and sums are chains of integer
+// instructions, and eight warps of 255 registers issued one instruction per cycle of the SM's four.  A norm without a class
+// (NaN, infinite) makes the leaf NaN.
+constexpr int kUmmaThreads = 512;
+template <int D, int INTEG>
+__device__ __forceinline__ void large_body_fx(const FusedParams &p, longlong2 *ws, int blk, int nblk, unsigned char *smem,
+                                              umma::Ctx &uc) {
+    constexpr int DD = D * D, NT = kUmmaThreads;
+    using fx::i64;
+    __shared__ int s_code, s_bad;
+    double *gam = (double *)(smem + large_front_bytes<double, D, 6>());
+    const double *packed = (const double *)p.packed;
+    const int tid = threadIdx.x, nb = p.n_basis, ext = fxl::extent(p.d_out);
+    const int ti = tid >> 4, tj = tid & 15;  // element passes: rows of 16 threads, no divisions by ext
+    longlong2 *SX = ws, *SX2 = ws + DD, *SX3 = ws + 2 * DD, *SR = ws + 3 * DD, *P0 = ws + 4 * DD, *P1 = ws + 5 * DD;
+    constexpr int GLD = D <= 128 ? D + 1 : D;  // packed exponent in the idle operand stages when it fits
+
+    const int64_t j0 = p.n_steps * blk / nblk;
+    const int len = (int)(p.n_steps * (blk + 1) / nblk - j0);
+    const bool traj = p.traj_out != nullptr;
+    if (tid == 0) s_bad = 0;
+    __syncthreads();
+    for (int i = ti; i < ext; i += NT / 16)
+        for (int jj = tj; jj < ext; jj += 16) {
+            const int e = i * D + jj;
+            longlong2 v = make_longlong2(i == jj ? 1ll << fx::F : 0, 0);
+            if (traj) {
+                const double2 x = p.traj_pin[(size_t)blk * DD + e];
+                v = make_longlong2(fx::from_double(x.x, 0), fx::from_double(x.y, 0));
+                if (!(fabs(x.x) < 2.0 && fabs(x.y) < 2.0)) s_bad = 1;
+            }
+            SR[e] = v;
+        }
+    unsigned flags = 0;
+    unsigned long long n_exp = 0;
+    int m_max = 0, s_max = 0;
+
+    for (int t = 0; t < len; ++t) {
+        const int64_t j = j0 + t;
+        if (tid == 0) {
+            slice_coefficients<double, INTEG, 1>(p, j, true, gam);
+            double nu = 0.0;
+            for (int e = 0; e < nb; ++e) nu = fma(fabs(gam[e]), p.bnorm1[e], nu);
+            s_code = p.cls_code[find_class(p, nu, &flags)];
+            if (flags) s_bad = 1;
+        }
+        __syncthreads();
+        const int code = s_code;
+        const double bad = s_bad ? nan("") : 0.0;
+        const int q = cls_q(code), rh = cls_r(code), s = cls_s(code) + p.extra_squarings;
+        double *gpk = D <= 128 ? (double *)smem : (double *)P0;
+        // packed exponent sum_b gamma_b P_b, two columns per thread
+        for (int i = ti; i < ext; i += NT / 16)
+            for (int jj = 2 * tj; jj < ext; jj += 32) {
+                double v0 = 0.0, v1 = 0.0;
+#pragma unroll 4
+                for (int b = 0; b < nb; ++b) {
+                    const double2 w = *reinterpret_cast<const double2 *>(packed + (size_t)b * DD + i * D + jj);
+                    v0 = fma(gam[b], w.x, v0);
+                    v1 = fma(gam[b], w.y, v1);
+                }
+                gpk[i * GLD + jj] = v0;
+                gpk[i * GLD + jj + 1] = v1;
+            }
+        __syncthreads();
+        // X = -i G / 2^s (upper triangle: Re G, strict lower: Im G)
+        for (int i = ti; i < ext; i += NT / 16)
+            for (int jj = tj; jj < ext; jj += 16) {
+                const i64 a = fx::from_double(gpk[i * GLD + jj], s), b = fx::from_double(gpk[jj * GLD + i], s);
+                const i64 re = (i <= jj) ? a : b, im = (i > jj) ? a : ((i < jj) ? -b : 0);
+                SX[i * D + jj] = make_longlong2(im, -re);
+            }
+        __syncthreads();
+        auto mm = [&](const longlong2 *A, const longlong2 *B, longlong2 *O) {
+            fxu::cta_mm<D, NT, longlong2>(A, B, O, smem, p.d_out, uc);
+        };
+        if (q >= 2) mm(SX, SX, SX2);
+        if (q >= 3) mm(SX2, SX, SX3);
+        const longlong2 *Xq = (q == 1) ? SX : ((q == 2) ? SX2 : SX3);
+        // T = (top ? a_{q rh} : 1) src + B_b, B_b = a_{q b} I + a_{q b + 1} X + a_{q b + 2} X^2 (q terms), a_k = 1 / k!
+        auto add_block = [&](longlong2 *T, const longlong2 *src, bool top, int b) {
+            const i64 a0 = fx::c_inv_fx[q * b];
+            const fx::Coef ct = fx::c_inv[q * rh], c1 = fx::c_inv[q * b + 1], c2 = fx::c_inv[q * b + 2];
+            const bool half = top && q * rh == 2, scaled = top && q * rh > 2;
+            for (int i = ti; i < ext; i += NT / 16)
+                for (int jj = tj; jj < ext; jj += 16) {
+                    const int e = i * D + jj;
+                    longlong2 v = src[e];
+                    if (scaled) v = make_longlong2(fx::mulc(v.x, ct), fx::mulc(v.y, ct));
+                    if (half) v = make_longlong2(fx::halve(v.x), fx::halve(v.y));
+                    if (i == jj) v.x += a0;
+                    if (q >= 2) {
+                        const longlong2 x = SX[e];
+                        v.x += b == 0 ? x.x : fx::mulc(x.x, c1);
+                        v.y += b == 0 ? x.y : fx::mulc(x.y, c1);
+                    }
+                    if (q >= 3) {
+                        const longlong2 x = SX2[e];
+                        v.x += b == 0 ? fx::halve(x.x) : fx::mulc(x.x, c2);
+                        v.y += b == 0 ? fx::halve(x.y) : fx::mulc(x.y, c2);
+                    }
+                    T[e] = v;
+                }
+            __syncthreads();
+        };
+        longlong2 *cur = P0, *nxt = P1;
+        auto swap = [](longlong2 *&a, longlong2 *&b) {
+            longlong2 *x = a;
+            a = b;
+            b = x;
+        };
+        add_block(cur, Xq, true, rh - 1);
+        for (int b = rh - 2; b >= 0; --b) {
+            mm(Xq, cur, nxt);
+            add_block(nxt, nxt, false, b);
+            swap(cur, nxt);
+        }
+        for (int i = 0; i < s; ++i) {
+            mm(cur, cur, nxt);
+            swap(cur, nxt);
+        }
+        mm(cur, SR, nxt);  // leaf product R <- U_j R into the free buffer, which becomes R
+        longlong2 *old = SR;
+        SR = nxt;
+        P0 = cur;
+        P1 = old;
+
+        if (traj && ((j + 1) % p.traj_every == 0 || j + 1 == p.n_steps)) {
+            const int64_t o = j / p.traj_every;
+            const int d = p.d_out;
+            if (p.traj_psi0 == nullptr) {
+                for (int e = tid; e < d * d; e += NT) {
+                    const longlong2 v = SR[(e / d) * D + e % d];
+                    const size_t at = (size_t)o * d * d + e;
+                    const double re = fx::to_double(v.x) + bad, im = fx::to_double(v.y) + bad;
+                    if (p.out_c128) ((double2 *)p.traj_out)[at] = make_double2(re, im);
+                    else ((float2 *)p.traj_out)[at] = make_float2((float)re, (float)im);
+                }
+            } else {
+                for (int i = tid; i < d; i += NT) {
+                    double re = bad, im = bad;
+                    for (int k = 0; k < d; ++k) {
+                        const longlong2 a = SR[i * D + k];
+                        const double2 b = p.traj_psi0[k];
+                        const double ax = fx::to_double(a.x), ay = fx::to_double(a.y);
+                        re = fma(ax, b.x, fma(-ay, b.y, re));
+                        im = fma(ax, b.y, fma(ay, b.x, im));
+                    }
+                    const size_t at = (size_t)o * d + i;
+                    if (p.out_c128) ((double2 *)p.traj_out)[at] = make_double2(re, im);
+                    else ((float2 *)p.traj_out)[at] = make_float2((float)re, (float)im);
+                }
+            }
+        }
+        if (tid == 0) {
+            n_exp += (unsigned long long)((q - 1) + (rh - 1) + s);
+            m_max = max(m_max, cls_m(code));
+            s_max = max(s_max, s);
+        }
+    }
+    __syncthreads();
+    if (traj) return;  // the forward pass combined the leaves and recorded the statistics
+
+    if (tid == 0 && len > 0) {
+        atomicAdd(&p.counters[0], n_exp);
+        atomicAdd(&p.counters[1], (unsigned long long)len);
+        atomicMax(&p.counters[2], (unsigned long long)m_max);
+        atomicMax(&p.counters[3], (unsigned long long)s_max);
+    }
+    if (flags) atomicOr(&p.status[0], flags);
+    // block partial (the leaf product) as doubles, the identity beyond the dimension
+    const double bad = s_bad ? nan("") : 0.0;
+    for (int e = tid; e < DD; e += NT) {
+        double2 v = make_double2((e / D) == (e % D) ? 1.0 : 0.0, 0.0);
+        if (max(e / D, e % D) < p.d_out) v = make_double2(fx::to_double(SR[e].x) + bad, fx::to_double(SR[e].y) + bad);
+        p.partials[(size_t)blk * DD + e] = v;
+        if (p.leaf_out) p.leaf_out[(size_t)blk * DD + e] = v;
+        if (p.block_out) p.block_out[(size_t)blk * DD + e] = v;
     }
     __threadfence();
     __syncthreads();
@@ -594,7 +790,7 @@ __host__ __device__ constexpr int large_min_blocks() {
 }
 
 template <typename Real, int D, int INTEG, int TC = 0>
-__global__ void __launch_bounds__(kLargeThreads, large_min_blocks<Real, D, TC>())
+__global__ void __launch_bounds__(large_tcm<Real, D, TC>() == 6 ? kUmmaThreads : kLargeThreads, large_min_blocks<Real, D, TC>())
     large_kernel(const FusedParams p, void *scratch) {
     extern __shared__ __align__(16) unsigned char smem[];
     using C = typename Cx<Real>::T;
@@ -615,12 +811,20 @@ __global__ void __launch_bounds__(kLargeThreads, large_min_blocks<Real, D, TC>()
         __shared__ int s_abort;
         umma::Ctx cx;
         umma::setup(cx, s_mbar, &s_tmem, &s_abort, p.status);
-        large_body<Real, D, INTEG, TCM>(p, ws, blockIdx.x, gridDim.x, smem, &cx);
+        if constexpr (TCM == 6) large_body_fx<D, INTEG>(p, (longlong2 *)ws, blockIdx.x, gridDim.x, smem, cx);
+        else large_body<Real, D, INTEG, TCM>(p, ws, blockIdx.x, gridDim.x, smem, &cx);
         umma::teardown(cx);
     } else {
         large_body<Real, D, INTEG, TCM>(p, ws, blockIdx.x, gridDim.x, smem);
     }
     // the pairwise tree over the block partials runs in tree_level_kernel launches
+}
+
+// FP64, D >= 64 with the Chebyshev exponential, whose recurrence leaves the fixed-point range: products on the FP64 pipe
+template <int D, int INTEG>
+__global__ void __launch_bounds__(kLargeThreads, 1) large_cheb_kernel(const FusedParams p, void *scratch) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    large_body<double, D, INTEG, 0>(p, (double2 *)scratch + (size_t)blockIdx.x * kLargeSlots * D * D, blockIdx.x, gridDim.x, smem);
 }
 
 // Pairwise tree over the nblk leaf products of one problem without waiting:
@@ -862,9 +1066,14 @@ cudaError_t leaf_prefixes(const double2 *leaf, int n, int d, double2 *a, double2
 template <typename Real, int D, int INTEG, int TC = 0>
 cudaError_t launch_large(const FusedParams &p, void *scratch, int grid, size_t smem, cudaStream_t st) {
     auto k = large_kernel<Real, D, INTEG, TC>;
+    int threads = kLargeThreads;
+    if constexpr (large_tcm<Real, D, TC>() == 6) {
+        if (p.cheb_m != nullptr) k = large_cheb_kernel<D, INTEG>;
+        else threads = kUmmaThreads;
+    }
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, kLargeThreads, smem, st>>>(p, scratch);
+    k<<<grid, threads, smem, st>>>(p, scratch);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (p.traj_out) return cudaSuccess;  // trajectory pass: no tree
     if ((e = allow_block_mm_smem(tree_level_fx_kernel<D>)) != cudaSuccess) return e;
