@@ -1,21 +1,21 @@
 // FP64-grade complex products of D >= 64 matrices on the digit products (pm_digits.cuh) with tcgen05: the 5th-generation
 // tensor cores multiply f16 digits four times as fast as mma.sync, asynchronously, and keep the sums in tensor memory.
 //
-// Per 64 x 64 output block one chain of M = 128, N = 64, K = 16 MMAs forms Re and Im at once,
+// Per 64 x 64 output block one chain of M = 128, K = 16 MMAs forms Re and Im at once,
 //   [[Ar, -Ai], [Ai, Ar]] [Br; Bi]:  tensor-memory lanes 0..63 the rows of Re C, 64..127 those of Im C,
 // with one f32 accumulator of 64 columns for each diagonal i + j = t of digit pairs (t = 0..7: all 512 columns).
 // Up to 128 real terms (64 complex k) the sums are integers below 2^24, hence exact; longer products are read back
-// every 64 k.  Warps 1..7 convert a panel of 16 k of both operands to fixed point and store its digits as f16 in the
+// every 64 k.  All warps convert a panel of 16 k of both operands to fixed point and store its digits as f16 in the
 // canonical no-swizzle K-major layout (A: planes -Ai, Ar, Ai per digit, so both halves of the embedding are 128 consecutive
-// rows; B: Br of every digit, then Bi), while thread 0 issues the 24 MMAs of the panel before; then all warps read the accumulators back,
-// add the diagonals in 64-bit integers and round to doubles.
+// rows; B: Br of every digit, then Bi) beside the MMAs of the panel before, which thread 0 issued (24 of them); then all
+// warps read the accumulators back, add the diagonals in 64-bit integers and round.
 //
 // Bound by the integer instructions that split the operands and sum the diagonals, not by the MMAs (64 x 64 x 64: 96 MMAs,
 // 8.7 k cycles at 4096 multiply-adds per cycle).  Blocks of 64 x 64 because the eight diagonals fill the tensor memory at
 // 64 columns.  Measured (d = 40, N = 4000 / d = 128, N = 608; on the FP64 pipe 61 / 86 ms, mma.sync products of pm_fxl.cuh
 // 7.0 / 13.4 ms): one MMA per digit pair, eight warps, doubles in and out 5.2 / 8.9 ms; sixteen warps 4.6 / 7.8 ms; up to
 // four pairs per MMA (one thread issued 68 per panel, now 24) 3.9 / 7.2 ms; fixed-point operands and results
-// (large_body_fx) 2.7 / 5.5 ms.  At D = 32 an M = 128 tile would be half padding: pm_fxl.cuh stays there, in the trees and
+// (large_body_fx) 2.73 / 5.49 ms; the next panel converted by all warps beside the MMAs 2.70 / 5.28 ms.  At D = 32 an M = 128 tile would be half padding: pm_fxl.cuh stays there, in the trees and
 // in the batched kernel (whose tensor memory belongs to its 3xTF32 products).
 //
 // Entries must be below 2 in magnitude; a NaN, an infinity or a larger entry makes the output block NaN.  Waits are
@@ -80,7 +80,7 @@ __device__ __forceinline__ void result(i64 q, bool, i64 &v) { v = (q + 7 + ((q >
 template <int NT, typename E>
 __device__ __forceinline__ void block_mm(const E *A, int lda, const E *B, int ldb, E *C, int ldc, int K,
                                          int rows, int cols, unsigned char *smem, umma::Ctx &cx) {
-    constexpr int kProducers = NT - 32, PER = (ITEMS + kProducers - 1) / kProducers;
+    constexpr int PER = ITEMS / NT;   // pairs per thread and panel
     constexpr int W = 64 * 128 / NT;  // accumulator columns per warp
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (*(volatile int *)cx.abort) return;  // uniform: set before the last block barrier
@@ -91,14 +91,14 @@ __device__ __forceinline__ void block_mm(const E *A, int lda, const E *B, int ld
     auto load = [&](int k0) {
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
-            const int it = tid - 32 + kProducers * i, w = it & 511;
+            const int it = tid + NT * i, w = it & 511;
             const int r = 8 * (w >> 6) + ((w >> 2) & 7), k = k0 + 8 * ((w >> 5) & 1) + 2 * (w & 3);
             if (it < 512) {
                 if (r < rows) {
                     v[i][0] = A[(size_t)r * lda + k];
                     v[i][1] = A[(size_t)r * lda + k + 1];
                 }
-            } else if (it < ITEMS && r < cols) {
+            } else if (r < cols) {
                 v[i][0] = B[(size_t)k * ldb + r];
                 v[i][1] = B[(size_t)(k + 1) * ldb + r];
             }
@@ -108,8 +108,8 @@ __device__ __forceinline__ void block_mm(const E *A, int lda, const E *B, int ld
         unsigned char *st = smem + (size_t)buf * STAGE;
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
-            const int it = tid - 32 + kProducers * i, w = it & 511, r = 8 * (w >> 6) + ((w >> 2) & 7);
-            if (it >= ITEMS || r >= (it < 512 ? rows : cols)) continue;
+            const int it = tid + NT * i, w = it & 511, r = 8 * (w >> 6) + ((w >> 2) & 7);
+            if (r >= (it < 512 ? rows : cols)) continue;
             uint32_t re[ND], im[ND];
             fx::split_pair(fixed(v[i][0].x, bad), fixed(v[i][1].x, bad), re);
             fx::split_pair(fixed(v[i][0].y, bad), fixed(v[i][1].y, bad), im);
@@ -161,22 +161,26 @@ __device__ __forceinline__ void block_mm(const E *A, int lda, const E *B, int ld
 
     const int np = K / KP;
     uint32_t used[2] = {cx.cnt[umma::kBarDone], cx.cnt[umma::kBarDone + 1]};  // completions before panel p of each stage
-    if (warp != 0) load(0);
+    auto stage = [&](int p) {  // panel p into its stage, panel p + 1 on its way
+        store(p & 1);
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        if (p + 1 < np) load((p + 1) * KP);
+    };
+    load(0);
+    stage(0);
+    any = __syncthreads_or(bad);
     for (int p = 0; p < np; ++p) {
         const int buf = p & 1;
-        if (warp != 0) {
-            if (p >= 2) umma::wait_idx(cx, umma::kBarDone + buf, used[buf] + p / 2 - 1);
-            store(buf);
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            if (p + 1 < np) load((p + 1) * KP);
-        }
-        any = __syncthreads_or(bad) || any;
         if (tid == 0) {
             umma::fence_after();
             issue(buf, (p * KP) % KMAX == 0);
             umma::commit(cx.bar + umma::kBarDone + buf);
         }
         __syncwarp();
+        if (p + 1 < np) {  // beside the MMAs of panel p, once those of panel p - 1 have left the stage
+            if (p >= 1) umma::wait_idx(cx, umma::kBarDone + (buf ^ 1), used[buf ^ 1] + (p - 1) / 2);
+            stage(p + 1);
+        }
         if (p + 1 == np || ((p + 1) * KP) % KMAX == 0) {  // read back
             umma::wait_idx(cx, umma::kBarDone + buf, used[buf] + p / 2);
             umma::fence_after();
@@ -194,8 +198,8 @@ __device__ __forceinline__ void block_mm(const E *A, int lda, const E *B, int ld
                 }
             }
             umma::fence_before();
-            if (p + 1 < np) __syncthreads();  // every accumulator is read before the next part starts
         }
+        any = __syncthreads_or(bad) || any;  // panel p + 1 is staged, and every accumulator read before a next part starts
     }
     cx.cnt[umma::kBarDone] += (np + 1) / 2;
     cx.cnt[umma::kBarDone + 1] += np / 2;
