@@ -79,7 +79,10 @@ typedef enum {
 
 /*
  * Arithmetic of the exponential and of the product tree.
- *  FP64: everything in double.
+ *  FP64: double inputs, results and coefficients.  d >= 5: the complex products and the exponents run in 64-bit fixed
+ *        point with exact sums (tensor cores, base-256 digits; absolute rounding 2^-57 on matrices of norm about one,
+ *        the size of a double's rounding there); d <= 4, the Chebyshev option, batched items of d <= 16 and
+ *        parament_propagate_noalloc: double arithmetic throughout.
  *  FP32: exponent assembly, exponential and the in-block tree in float; the
  *        norm bound that picks the Taylor degree and the number of squarings,
  *        and the product tree above the thread-block level, in double.
@@ -115,7 +118,7 @@ typedef enum {
     /* thread blocks of the fused kernel; 0 (default) = fill every SM */
     PARAMENT_OPT_GRID_BLOCKS = 2,
     /* warps per thread block; 0 (default) = largest that fits shared memory (at most 16 for FP32
-       d in 9..16, 8 otherwise) */
+       d in 9..16, 16 for FP64 d in 5..8, 8 otherwise; d <= 2: 4, or what a single block needs) */
     PARAMENT_OPT_BLOCK_WARPS = 3,
     /* 1 (default) = reject non-Hermitian H in set_hamiltonians; 0 = skip the check */
     PARAMENT_OPT_CHECK_HERMITIAN = 4,
@@ -124,11 +127,12 @@ typedef enum {
     /* Hermiticity tolerance in units of 1e-12 relative to max |H_ab| (default 1000, i.e. 1e-9) */
     PARAMENT_OPT_HERMITIAN_TOL_E12 = 7,
     /* gradient: slices per sub-chunk of the adjoint sweep (0 = auto: a whole leaf when it fits the
-       workspace cap); leaves longer than a sub-chunk are re-computed from checkpoints */
+       workspace cap); leaves longer than a sub-chunk are re-computed from checkpoints.  FP64 with d >= 5 keeps
+       no prefixes: reported, without effect */
     PARAMENT_OPT_GRAD_SUBCHUNK = 8,
     /* gradient: cap in MiB on the per-slice prefix buffer of the adjoint sweep (default 4096) */
     PARAMENT_OPT_WORKSPACE_MB = 9,
-    /* batched: target slices per leaf (0 = default 64) */
+    /* batched: target slices per leaf (0 = by dimension: 8 for d > 16, 16 for d in 9..16, else 64) */
     PARAMENT_OPT_BATCH_LEAF_STEPS = 10,
     /* batched: work items per SM (0 = default 32) */
     PARAMENT_OPT_BATCH_ITEMS_PER_SM = 11,
@@ -171,8 +175,9 @@ typedef struct {
 
 /* product back-ends reported in parament_stats.product_backends (a batched call ORs the
    back-ends of its dimension classes) */
-#define PARAMENT_BACKEND_CUDA_CORES 0x1u /* FP32 / FP64 fused multiply-adds */
-#define PARAMENT_BACKEND_MMA_SYNC 0x2u   /* warp-level mma.sync instructions (no path of this build uses them) */
+#define PARAMENT_BACKEND_CUDA_CORES 0x1u /* the precision's own arithmetic: FP32 / FP64 fused multiply-adds, or the
+                                            exact integer-digit products of FP64 */
+#define PARAMENT_BACKEND_MMA_SYNC 0x2u   /* reduced-precision products by warp-level mma.sync (no path of this build) */
 #define PARAMENT_BACKEND_TCGEN05 0x4u    /* tcgen05.mma with tensor-memory accumulators */
 
 #define PARAMENT_DEV_NONFINITE_NORM 0x1u /* a slice's norm bound was NaN/Inf */
@@ -254,7 +259,8 @@ int parament_propagate(parament_ctx *ctx, void *U_out, parament_precision prec);
  * as the upper-right block of exp([[X, Lambda], [0, X]]).  The prefixes P and suffixes S come from
  * the forward tree: leaf and block products of the forward kernel, exclusive scans over them, then
  * per leaf a forward sweep (prefixes, re-computed from checkpoints for long leaves) and a backward
- * sweep.  A Simpson end sample belongs to two slices and receives both contributions.  d <= 16:
+ * sweep; FP64 of d >= 5 undoes the slices in one backward sweep instead, and FP32 of d = 5..8 up to 2048
+ * slices is computed in FP64 and rounded.  A Simpson end sample belongs to two slices and receives both contributions.  d <= 16:
  * groups of lanes of one warp per leaf; d = 17..256: one thread block per leaf (FP64 Hillis-Steele
  * scans of the leaf products for the prefixes, the suffixes, U(T) and z; block-wide products).
  * V: d x d in the dtype of set_hamiltonians; U_out: optional U(T).  Pointers host or device.

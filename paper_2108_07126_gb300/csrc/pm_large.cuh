@@ -51,8 +51,9 @@ template <typename Real, int D> struct LGeo {
 };
 
 // TCM: 0 = CUDA-core products, 2 = 3xTF32 with tcgen05 (D = 128, 256: 128 x 128 output blocks),
-// 3 = split BF16x3 with tcgen05 (D = 128, 256), 6 = FP64 digit products with tcgen05 (D >= 64; FP64 with 0: mma.sync), 4 / 5 = 3xTF32 / split BF16x3 with tcgen05 in the
-// shared-memory body of pm_tc_small.cuh (D = 32, 64)
+// 3 = split BF16x3 with tcgen05 (D = 128, 256), 4 / 5 = 3xTF32 / split BF16x3 with tcgen05 in the
+// shared-memory body of pm_tc_small.cuh (D = 32, 64), 6 = FP64 digit products with tcgen05 (D >= 64,
+// large_body_fx; FP64 with 0: digit products on mma.sync)
 template <int TCM> __host__ __device__ constexpr int tcm_format() { return (TCM == 3 || TCM == 5) ? umma::kBF16x3 : umma::kTF32x3; }
 
 // FP64 levels of the arrival tree on the digit products in the FP32 kernels too: where their shared memory holds
