@@ -179,11 +179,13 @@ __global__ void __launch_bounds__(Cfg<D>::MAXW * 32, 1) fx_kernel(const FusedPar
     const int len = (int)(p.n_steps * (leaf + 1) / n_leaves - j0);
 
     Tile<D> T;
+    unsigned bad_prefix = 0;  // a prefix with a NaN (fixed point has none): every output of the leaf is NaN
 #pragma unroll
     for (int e = 0; e < NE; ++e) {  // R^T = I, or the prefix of the leaf
         const int j = L<D>::row(lane, e), i = L<D>::col(lane, e);
         if constexpr (TRAJ) {
             const double2 v = p.traj_pin[(size_t)leaf * DD + i * D + j];
+            bad_prefix |= !(fabs(v.x) < 2.0) || !(fabs(v.y) < 2.0);
             T.re[e] = from_double(v.x, 0);
             T.im[e] = from_double(v.y, 0);
         } else {
@@ -355,7 +357,7 @@ __global__ void __launch_bounds__(Cfg<D>::MAXW * 32, 1) fx_kernel(const FusedPar
                 if ((j + 1) % p.traj_every == 0 || j + 1 == p.n_steps) {
                     const int64_t o = j / p.traj_every;
                     const int d = p.d_out;
-                    const double bad = __any_sync(0xffffffffu, flags) ? nan("") : 0.0;
+                    const double bad = __any_sync(0xffffffffu, flags || bad_prefix) ? nan("") : 0.0;
                     if (p.traj_psi0 == nullptr) {
 #pragma unroll
                         for (int e = 0; e < NE; ++e) {
