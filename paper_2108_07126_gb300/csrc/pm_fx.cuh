@@ -199,16 +199,24 @@ __global__ void __launch_bounds__(Cfg<D>::MAXW * 32, 1) fx_kernel(const FusedPar
     unsigned flags = 0;
     unsigned long long n_exp = 0;
     int m_max = 0, s_max = 0;
+    // trajectory mode: the outputs of slices bad_from, bad_from + 1, ... of the leaf are NaN, those before it are valid
+    int bad_from = TRAJ && __any_sync(0xffffffffu, bad_prefix) ? 0 : len;
 
     for (int t0 = 0; t0 < len; t0 += kGT) {
         __syncwarp();
+        unsigned tile_flags = 0;
         if (lane < kGT) {
             const bool act = t0 + lane < len;
             double *gcol = gam + lane;
             slice_coefficients<double, INTEG, kGT>(p, j0 + t0 + lane, act, gcol);
             double nu = 0.0;
             for (int e = 0; e < nb; ++e) nu = fma(fabs(gcol[e * kGT]), bnorm[e], nu);
-            cls[lane] = find_class(p, nu, &flags);
+            cls[lane] = find_class(p, nu, &tile_flags);
+            flags |= tile_flags;
+        }
+        if constexpr (TRAJ) {
+            const unsigned m = __ballot_sync(0xffffffffu, tile_flags != 0);
+            if (m) bad_from = min(bad_from, t0 + __ffs(m) - 1);
         }
         __syncwarp();
         const int nr = min(kGT, len - t0);
@@ -357,7 +365,7 @@ __global__ void __launch_bounds__(Cfg<D>::MAXW * 32, 1) fx_kernel(const FusedPar
                 if ((j + 1) % p.traj_every == 0 || j + 1 == p.n_steps) {
                     const int64_t o = j / p.traj_every;
                     const int d = p.d_out;
-                    const double bad = __any_sync(0xffffffffu, flags || bad_prefix) ? nan("") : 0.0;
+                    const double bad = t0 + rr >= bad_from ? nan("") : 0.0;
                     if (p.traj_psi0 == nullptr) {
 #pragma unroll
                         for (int e = 0; e < NE; ++e) {

@@ -17,6 +17,8 @@
 // t_e = Im Tr(M B_e); the traces of sixteen slices are one digit GEMM against the basis.
 #pragma once
 
+#include <climits>
+
 #include "pm_fx.cuh"
 #include "pm_grad.cuh"
 
@@ -147,13 +149,16 @@ __global__ void __launch_bounds__(kScanWarps * 32) fx_group_kernel(const double2
 }
 
 // Exclusive prefixes (blockIdx.y = 0) or suffixes (1) of the leaves of forward block blockIdx.x; the prefix block of
-// the last forward block also writes U(T) (pin[L], U_out), z and the loss.
+// the last forward block also writes U(T) (pin[L], U_out), z and the loss.  A bad leaf (NaN, which fixed point has not) makes
+// the elements that contain it NaN: the prefixes of later leaves, the suffixes of earlier ones.
 template <int D>
 __global__ void __launch_bounds__(kScanWarps * 32) fx_scan_kernel(const ScanParams sp, const double2 *groups) {
     constexpr int NT = L<D>::NE * 32, DD = D * D;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x, n = sp.n_blocks, nl = sp.leaves_per_block;
     const bool suf = blockIdx.y != 0;
+    __shared__ int s_bad;  // the bad element nearest to the seed
+    if (threadIdx.x == 0) s_bad = suf ? -1 : INT_MAX;
     longlong2 *tiles = (longlong2 *)smem;
     uint32_t *rhs = (uint32_t *)(smem + (size_t)ScanSmem<D>::MAXE * ScanSmem<D>::TILE + (size_t)warp * ScanSmem<D>::RHS);
     const int gb = b / kGroup, ng = (n + kGroup - 1) / kGroup;
@@ -166,7 +171,7 @@ __global__ void __launch_bounds__(kScanWarps * 32) fx_scan_kernel(const ScanPara
         block_chain<D>(in + ng - 1 - gb, [&](int i) { return i < in ? sp.blockpart + (size_t)(b + 1 + i) * DD : groups + (size_t)(gb + 1 + i - in) * DD; },
                        tiles, rhs, lane, warp, bad);
     }
-    __syncthreads();
+    const bool seed_bad = __syncthreads_or((int)bad) != 0;
     // elements: prefix x_0 = seed, x_l = leaf_{l-1} (one more for U(T)); suffix x_{nl-1} = seed, x_l = leaf_{l+1}
     const double2 *leaf = sp.leafpart + (size_t)b * nl * DD;
     const bool last = !suf && b == n - 1;
@@ -181,10 +186,15 @@ __global__ void __launch_bounds__(kScanWarps * 32) fx_scan_kernel(const ScanPara
     }
     for (int l = warp; l < ne; l += kScanWarps) {
         if (l == (suf ? nl - 1 : 0)) continue;
+        bad = 0;
         ld_transposed<D>(leaf + (size_t)(suf ? l + 1 : l - 1) * DD, lane, t, bad);
         st_priv<D>(tiles + (size_t)l * NT, lane, t);
+        if (bad) {
+            if (suf) atomicMax(&s_bad, l);
+            else atomicMin(&s_bad, l);
+        }
     }
-    const unsigned any = (unsigned)__syncthreads_or((int)bad);
+    __syncthreads();
     constexpr int PER = (ScanSmem<D>::MAXE + kScanWarps - 1) / kScanWarps;
     for (int off = 1; off < ne; off <<= 1) {
         Tile<D> r[PER];
@@ -205,7 +215,7 @@ __global__ void __launch_bounds__(kScanWarps * 32) fx_scan_kernel(const ScanPara
     double2 *out = (suf ? sp.sout : sp.pin) + (size_t)b * nl * DD;
     for (int l = warp; l < ne; l += kScanWarps) {
         ld_priv<D>(tiles + (size_t)l * NT, lane, t);
-        st_doubles<D>(out + (size_t)l * DD, lane, t, any);
+        st_doubles<D>(out + (size_t)l * DD, lane, t, seed_bad || (suf ? l <= s_bad : l >= s_bad));
     }
     if (!last) return;
     __syncthreads();

@@ -53,3 +53,33 @@ def test_trajectory_is_nan_from_the_sample_on(prop, d, prec, grid, with_psi):
     _, _, _, out = trajectory_with_nan(prop, d, prec, grid, with_psi)
     after = out[BAD // EVERY:]  # outputs at slices EVERY (o + 1) > BAD, and the last
     assert np.isnan(after.real).all() and np.isnan(after.imag).all()
+
+
+@pytest.mark.parametrize("grid", [0, 2])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("d", [8, 12, 16, 24, 40])
+@pytest.mark.parametrize("with_psi", [False, True])
+def test_trajectory_before_the_sample_is_valid(prop, d, prec, grid, with_psi):
+    """The outputs before the sample equal the oracle's of the run that ends there."""
+    (H0, Hk, c), dt, psi, out = trajectory_with_nan(prop, d, prec, grid, with_psi)
+    n = BAD // EVERY
+    R = oracle.trajectory(H0, Hk, c[:, :n * EVERY], dt, "midpoint", EVERY)
+    if psi is not None:
+        R = R @ psi.numpy().astype(np.complex128)
+    err = np.max(np.abs(out[:n].astype(np.complex128) - R))
+    assert err <= (TOL64 if prec == "fp64" else tol32(d, n * EVERY))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("d", [8, 16, 24, 40])
+def test_gradient_is_nan_everywhere(prop, d, prec):
+    """Every component of the gradient depends on U(T), and so on every sample."""
+    import torch
+
+    prob = wl.random_problem(d, 2, 400, "midpoint", seed=6100 + d, g_norm=0.3)
+    prob.c[0, 133] = np.nan
+    hd, cd = (torch.complex128, torch.float64) if prec == "fp64" else (torch.complex64, torch.float32)
+    prop.set_hamiltonians(torch.as_tensor(prob.H0).to(hd), torch.as_tensor(prob.Hk).to(hd), prob.integrator)
+    prop.set_controls(torch.as_tensor(prob.c).to(cd), prob.dt, prob.n_steps)
+    loss, g = prop.propagate_grad(torch.eye(d, dtype=hd), prec)
+    assert np.isnan(loss) and torch.isnan(g).all()
