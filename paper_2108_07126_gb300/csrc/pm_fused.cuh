@@ -407,7 +407,15 @@ __device__ __forceinline__ void fused_body(const FusedParams &p, int blk, int nb
             if (EXPM != 1) {
                 double nu = 0.0;
                 for (int e = 0; e < nb; ++e) nu = fma(fabs((double)gcol[e * 32]), bnorm[e], nu);
-                cls[lane] = find_class(p, nu, &flags);
+                // the groups of a warp share the highest class of their slices: a slice without a finite norm is NaN in
+                // any class, and the top one would put its squarings' rounding (1e-8 at d = 2, FP64) on the others
+                if (GPW > 1 && !isfinite(nu)) {
+                    flags |= kDevNonfinite;
+                    for (int e = 0; e < nb; ++e) gcol[e * 32] = (Real)nan("");
+                    cls[lane] = 0;
+                } else {
+                    cls[lane] = find_class(p, nu, &flags);
+                }
             } else {
                 cls[lane] = 0;  // Chebyshev: one global degree, fixed before the launch
             }

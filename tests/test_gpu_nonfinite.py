@@ -25,8 +25,8 @@ def prop():
 N, BAD, EVERY = 1203, 619, 7  # BAD: slice of the sample, inside a tile and a leaf for every geometry below
 
 
-def trajectory_with_nan(prop, d, prec, grid, with_psi):
-    """(problem with rounded inputs, psi_0 or None, output) of a run whose slice BAD has a NaN sample."""
+def trajectory_with_nan(prop, d, prec, grid, with_psi, bad=BAD, value=float("nan")):
+    """(rounded inputs, dt, psi_0 or None, output) of a run whose slice `bad` has a non-finite sample."""
     import torch
 
     from paper_2108_07126_gb300 import binding as b
@@ -35,7 +35,7 @@ def trajectory_with_nan(prop, d, prec, grid, with_psi):
     hd, cd = (torch.complex128, torch.float64) if prec == "fp64" else (torch.complex64, torch.float32)
     H0, Hk, c = torch.as_tensor(prob.H0).to(hd), torch.as_tensor(prob.Hk).to(hd), torch.as_tensor(prob.c).to(cd)
     psi = torch.as_tensor(wl.haar_unitary(np.random.default_rng(6001 + d), d)[:, 0].copy()).to(hd) if with_psi else None
-    c[1, BAD] = float("nan")
+    c[1, bad] = value
     prop.set_option(b.PARAMENT_OPT_GRID_BLOCKS, grid)
     prop.set_hamiltonians(H0, Hk, prob.integrator)
     prop.set_controls(c, prob.dt, N)
@@ -68,6 +68,19 @@ def test_trajectory_before_the_sample_is_valid(prop, d, prec, grid, with_psi):
         R = R @ psi.numpy().astype(np.complex128)
     err = np.max(np.abs(out[:n].astype(np.complex128) - R))
     assert err <= (TOL64 if prec == "fp64" else tol32(d, n * EVERY))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("bad", [50, 619, 1000])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_other_leaves_of_the_warp_keep_their_class(prop, d, prec, bad, value):
+    """d <= 8: several leaves per warp, whose slices share the degree and the squarings of the highest norm."""
+    (H0, Hk, c), dt, _, out = trajectory_with_nan(prop, d, prec, 0, False, bad, value)
+    n = bad // EVERY
+    R = oracle.trajectory(H0, Hk, c[:, :n * EVERY], dt, "midpoint", EVERY)
+    assert np.max(np.abs(out[:n].astype(np.complex128) - R)) <= (TOL64 if prec == "fp64" else tol32(d, n * EVERY))
+    assert np.isnan(out[n:].real).all() and np.isnan(out[n:].imag).all()
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
