@@ -156,7 +156,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32) su2_kernel(const FusedParams p
         }
         R = mul(Q<Real>{c, sc * x, sc * y, sc * z, (double)m}, R);
     }
-    if (p.unitary_step) {  // FP32: the Newton-Schulz step on a unit quaternion
+    // FP32: the Newton-Schulz step on a unit quaternion, on the block's product in double (below) and on leaves of more than 16
+    // slices.  The norm of a slice is exact to a rounding; it drifts in the products (Rabi qubit, N = 16384 in leaves of one
+    // slice: 2.7e-5 with the step on every leaf alone)
+    if (p.unitary_step && p.n_steps > 16 * n_leaves) {
         const Real f = Real(0.5) * (Real(3) - fma(R.a, R.a, fma(R.x, R.x, fma(R.y, R.y, R.z * R.z))));
         R.a *= f;
         R.x *= f;
@@ -177,6 +180,13 @@ __global__ void __launch_bounds__(kMaxWarps * 32) su2_kernel(const FusedParams p
     R = block_product(R, sm, W);
     __syncthreads();
     Q<double> U{(double)R.a, (double)R.x, (double)R.y, (double)R.z, R.ph};
+    if (p.unitary_step) {
+        const double f = 0.5 * (3.0 - fma(U.a, U.a, fma(U.x, U.x, fma(U.y, U.y, U.z * U.z))));
+        U.a *= f;
+        U.x *= f;
+        U.y *= f;
+        U.z *= f;
+    }
 
     if (gridDim.x > 1) {
         double *part = (double *)p.partials;

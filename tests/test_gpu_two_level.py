@@ -1,0 +1,45 @@
+"""Two-level systems (d <= 2) on unit quaternions: the FP32 norm correction."""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2108_07126_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture()
+def prop():
+    import torch
+
+    from paper_2108_07126_gb300.binding import Propagator
+
+    assert torch.cuda.is_available()
+    p = Propagator(0)
+    yield p
+    p.close()
+
+
+@pytest.mark.parametrize("n,grid,warps", [(2048, 0, 0), (16384, 0, 0), (16384, 1, 1), (3001, 3, 2), (100, 0, 0)])
+def test_fp32_norm_does_not_drift(prop, n, grid, warps):
+    """The Rabi qubit in leaves of one slice and of many.  Unitarity: a product of 128 slices has a norm off by at most
+    128 x 2^-22, which the step squares away; what is left is the rounding of U to complex64 (2^-24 an entry, 2^-22 with
+    room).  Error: below the 1.2e-5 of the 2 x 2 matrix products with a step on every leaf, measured at N = 2^14 (N = 100:
+    exponents of 31 radians, whose own rounding is larger)."""
+    import torch
+
+    from paper_2108_07126_gb300 import binding as b
+
+    prob = wl.rabi_qubit(n)
+    H0, Hk, c = prob.H0.astype(np.complex64), prob.Hk.astype(np.complex64), prob.c.astype(np.float32)
+    prop.set_option(b.PARAMENT_OPT_GRID_BLOCKS, grid)
+    prop.set_option(b.PARAMENT_OPT_BLOCK_WARPS, warps)
+    prop.set_hamiltonians(torch.as_tensor(H0), torch.as_tensor(Hk), prob.integrator)
+    prop.set_controls(torch.as_tensor(c), prob.dt, n)
+    U = prop.propagate("fp32").cpu().numpy().astype(np.complex128)
+    assert np.max(np.abs(U.conj().T @ U - np.eye(2))) <= 2.0 ** -22
+    if n < 2048:
+        return
+    R = oracle.propagate(H0.astype(np.complex128), Hk.astype(np.complex128), c.astype(np.float64), prob.dt, prob.integrator)
+    assert np.max(np.abs(U - R)) <= 1.2e-5
