@@ -113,7 +113,8 @@ typedef enum {
 /* keys of parament_set_option / parament_get_option */
 typedef enum {
     /* 0 (default) = choose the Taylor degree per slice from the norm bound;
-       m > 0 = force degree m (one of 1, 2, 4, 6, 9, 12), squarings still from the bound */
+       m > 0 = force degree m (one of 1, 2, 4, 6, 9, 12), squarings still from the bound.  U(T) of d <= 2 takes closed
+       forms of its own (cosine and sine of the rotation angle) unless a degree or extra squarings are set */
     PARAMENT_OPT_TAYLOR_DEGREE = 1,
     /* thread blocks of the fused kernel; 0 (default) = fill every SM */
     PARAMENT_OPT_GRID_BLOCKS = 2,
@@ -163,10 +164,10 @@ typedef struct {
     int32_t grid_blocks;      /* thread blocks launched */
     int32_t block_threads;    /* threads per block */
     int32_t leaves;           /* sequential leaf products below the pairwise tree */
-    int32_t max_degree;       /* largest Taylor degree used */
-    int32_t max_squarings;    /* largest number of squarings used */
+    int32_t max_degree;       /* largest Taylor degree used (U(T) of d <= 2: of the cosine and sine polynomials, 15 or 11) */
+    int32_t max_squarings;    /* largest number of squarings used (U(T) of d <= 2: doublings of the rotation angle) */
     int32_t grad_subchunk;    /* slices per sub-chunk of the latest gradient (0 if none) */
-    int64_t exp_products;     /* complex d x d products in exponentials and squarings */
+    int64_t exp_products;     /* complex d x d products in exponentials and squarings (U(T) of d <= 2: none) */
     int64_t tree_products;    /* complex d x d products in the product tree */
     uint32_t device_status;   /* PARAMENT_DEV_* bits raised by the kernels */
     uint32_t product_backends; /* PARAMENT_BACKEND_* bits: the code that ran the complex products */

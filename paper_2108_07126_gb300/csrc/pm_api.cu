@@ -1018,6 +1018,9 @@ int parament_set_controls(parament_ctx *ctx, const void *c, parament_real_dtype 
 
 namespace {
 
+// a forced Taylor degree or extra squarings: two-level systems take the matrix scheme, which has both
+bool matrix_scheme(const parament_ctx *ctx) { return ctx->opt_degree > 0 || ctx->opt_extra_sq > 0; }
+
 // Controls in the compute type, Taylor table and launch geometry of the fused
 // forward kernel (shared by propagate and propagate_grad).
 int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int &grid, int &warps, size_t &smem,
@@ -1068,7 +1071,7 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
     } else {
     const int max_warps = fused_max_warps(Dp, fp64, cheb);
     warps = (int)ctx->opt_warps;
-    const bool su2 = Dp == 2 && only_u;  // U(T) of a two-level system: one thread per leaf (pm_su2.cuh)
+    const bool su2 = Dp == 2 && only_u && !matrix_scheme(ctx);  // U(T) of a two-level system: one thread per leaf (pm_su2.cuh)
     if (warps <= 0 && su2) {
         // one block up to 256 slices (no tree between blocks), else blocks of 128 threads
         warps = ctx->n_steps <= 256 ? (int)std::max<int64_t>(1, (ctx->n_steps + 31) / 32) : 4;
@@ -1144,7 +1147,8 @@ cudaError_t forward_launch(parament_ctx *ctx, int fp64, const FusedParams &p, in
                            int tc = 0) {
     if (ctx->dpad > kMaxSmallDim)
         return large_dispatch(ctx->dpad, fp64, (int)ctx->integ, p, ctx->lscratch.ptr, grid, smem, ctx->stream, tc);
-    return fused_dispatch(ctx->dpad, fp64, (int)ctx->integ, p, grid, warps, smem, ctx->stream);
+    return fused_dispatch(ctx->dpad, fp64, (int)ctx->integ, p, grid, warps, smem, ctx->stream,
+                          ctx->dpad == 2 && matrix_scheme(ctx) ? 3 : 0);
 }
 
 void record_launch(parament_ctx *ctx, int nb, int grid, int warps, int leaves_per_block,

@@ -1,5 +1,6 @@
 // Instantiations of the fused propagation kernel for padded dimension 2
-// (mode cheb: 0 = Taylor exponential, 1 = Chebyshev exponential, 2 = Taylor trajectory).
+// (mode cheb: 0 = U(T) by unit quaternions, 1 = Chebyshev exponential, 2 = Taylor trajectory, 3 = Taylor exponential
+// with its degree and squarings).
 #include "pm_fused.cuh"
 #include "pm_su2.cuh"
 
@@ -8,8 +9,10 @@ namespace pm {
 cudaError_t fused_dispatch_d2(int fp64, int integ, const FusedParams &p, int grid, int warps, size_t smem,
                                cudaStream_t st, int cheb) {
     // U(T) alone: unit quaternions, one thread per leaf (a leaf per lane in the fused kernel too, so that the caller's
-    // geometry holds for both); the fused kernel where leaf or block products are kept
-    if (cheb == 0 && !p.leaf_out && !p.block_out) {
+    // geometry holds for both); the fused kernel where leaf or block products are kept or the degree is forced
+    if (cheb == 3) {
+        cheb = 0;
+    } else if (cheb == 0 && !p.leaf_out && !p.block_out) {
         switch (integ * 2 + (fp64 ? 1 : 0)) {
             case 0: return su2::launch<float, kMidpoint>(p, grid, warps, st);
             case 1: return su2::launch<double, kMidpoint>(p, grid, warps, st);

@@ -93,6 +93,8 @@ __device__ __forceinline__ void cos_sinc(float r2, float &c, float &s) {
 }
 
 constexpr int kMaxWarps = 8;
+// largest power of r in cos r and sin r as polynomials
+template <typename Real> __host__ __device__ constexpr int degree() { return sizeof(Real) == 8 ? 15 : 11; }
 
 template <typename Real, int INTEG>
 __global__ void __launch_bounds__(kMaxWarps * 32) su2_kernel(const FusedParams p) {
@@ -117,8 +119,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32) su2_kernel(const FusedParams p
     const int64_t j0 = p.n_steps * leaf / n_leaves;
     const int len = (int)(p.n_steps * (leaf + 1) / n_leaves - j0);
     Q<Real> R = identity<Real>();
-    unsigned flags = 0, n_exp = 0;
-    int m_max = 0, s_max = 0, cls = 0;
+    unsigned flags = 0;
+    int s_max = 0;
     Real gam[kMaxBasis];
     for (int t = 0; t < len; ++t) {
         slice_coefficients<Real, INTEG, 1>(p, j0 + t, true, gam);
@@ -132,12 +134,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32) su2_kernel(const FusedParams p
             m = fma(gam[e], (Real)b1.y, m);
             nu = fma(fabs((double)gam[e]), p.bnorm1[e], nu);
         }
-        // the class of the norm bound (statistics and status; neighbouring slices mostly share it)
-        if (!(nu <= p.cls_cap[cls] && (cls == 0 || nu > p.cls_cap[cls - 1]))) cls = find_class(p, nu, &flags);
-        const int code = p.cls_code[cls];
-        n_exp += (cls_q(code) - 1) + (cls_r(code) - 1) + cls_s(code) + p.extra_squarings;
-        m_max = max(m_max, cls_m(code));
-        s_max = max(s_max, cls_s(code) + p.extra_squarings);
+        find_class(p, nu, &flags);  // NaN, infinite and capped norms (the halvings follow r itself)
         // halve until r <= 1/2, double back
         Real r2 = fma(x, x, fma(y, y, z * z));
         int s = 0;
@@ -154,6 +151,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32) su2_kernel(const FusedParams p
             sc = Real(2) * c * sc;
             c = c2;
         }
+        s_max = max(s_max, s);
         R = mul(Q<Real>{c, sc * x, sc * y, sc * z, (double)m}, R);
     }
     // FP32: the Newton-Schulz step on a unit quaternion, on the block's product in double (below) and on leaves of more than 16
@@ -166,14 +164,13 @@ __global__ void __launch_bounds__(kMaxWarps * 32) su2_kernel(const FusedParams p
         R.y *= f;
         R.z *= f;
     }
-    // statistics
-    const unsigned we = __reduce_add_sync(0xffffffffu, n_exp), wl = __reduce_add_sync(0xffffffffu, (unsigned)len);
-    const int wm = __reduce_max_sync(0xffffffffu, m_max), ws = __reduce_max_sync(0xffffffffu, s_max);
+    // statistics (no matrix products in the exponentials)
+    const unsigned wl = __reduce_add_sync(0xffffffffu, (unsigned)len);
+    const int ws = __reduce_max_sync(0xffffffffu, s_max);
     const unsigned wf = __reduce_or_sync(0xffffffffu, flags);
     if (lane == 0) {
-        atomicAdd(&cnt[0], (unsigned long long)we);
         atomicAdd(&cnt[1], (unsigned long long)wl);
-        atomicMax(&cnt[2], (unsigned long long)wm);
+        if (wl) atomicMax(&cnt[2], (unsigned long long)degree<Real>());
         atomicMax(&cnt[3], (unsigned long long)ws);
         if (wf) atomicOr(&s_flags, wf);
     }

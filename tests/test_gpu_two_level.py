@@ -1,10 +1,11 @@
-"""Two-level systems (d <= 2) on unit quaternions: the FP32 norm correction."""
+"""Two-level systems (d <= 2) on unit quaternions: the FP32 norm correction, and the options of the matrix scheme."""
 
 import numpy as np
 import pytest
 
 import oracle
 from paper_2108_07126_gb300 import workloads as wl
+from tolerances import TOL64, tol32
 
 pytestmark = pytest.mark.gpu
 
@@ -43,3 +44,36 @@ def test_fp32_norm_does_not_drift(prop, n, grid, warps):
         return
     R = oracle.propagate(H0.astype(np.complex128), Hk.astype(np.complex128), c.astype(np.float64), prob.dt, prob.integrator)
     assert np.max(np.abs(U - R)) <= 1.2e-5
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("d", [1, 2])
+@pytest.mark.parametrize("degree,extra", [(0, 0), (4, 0), (12, 0), (0, 3), (9, 2)])
+def test_forced_degree_and_extra_squarings(prop, d, prec, degree, extra):
+    """Forced degrees and extra squarings run (the matrix scheme has them), and the statistics name what ran."""
+    import torch
+
+    from paper_2108_07126_gb300 import binding as b
+
+    n = 300
+    prob = wl.random_problem(d, 2, n, "magnus4_gl2", seed=6200 + d, g_norm=0.3)
+    hd, cd = (torch.complex128, torch.float64) if prec == "fp64" else (torch.complex64, torch.float32)
+    H0, Hk, c = torch.as_tensor(prob.H0).to(hd), torch.as_tensor(prob.Hk).to(hd), torch.as_tensor(prob.c).to(cd)
+    R = oracle.propagate(H0.numpy().astype(complex), Hk.numpy().astype(complex), c.numpy().astype(float), prob.dt,
+                         prob.integrator)
+    prop.set_option(b.PARAMENT_OPT_TAYLOR_DEGREE, degree)
+    prop.set_option(b.PARAMENT_OPT_EXTRA_SQUARINGS, extra)
+    prop.set_hamiltonians(H0, Hk, prob.integrator)
+    prop.set_controls(c, prob.dt, n)
+    U = prop.propagate(prec).cpu().numpy()
+    # every squaring doubles the rounding of the polynomial (a few 2^-53 a slice), and a low degree needs many
+    squarings = prop.stats()["max_squarings"]
+    tol = max(TOL64, 4 * n * 2.0 ** (squarings - 53)) if prec == "fp64" else tol32(d, n) * 2.0 ** squarings
+    assert np.max(np.abs(U - R)) <= tol
+    st = prop.stats()
+    assert st["tree_products"] == n and st["device_status"] == 0
+    if degree or extra:
+        assert st["max_degree"] == degree or degree == 0
+        assert squarings >= extra and st["exp_products"] >= n * extra
+    else:
+        assert st["exp_products"] == 0 and st["max_degree"] == (15 if prec == "fp64" else 11)
