@@ -19,7 +19,8 @@
 // in the batched kernel (whose tensor memory belongs to its 3xTF32 products).
 //
 // Entries must be below 2 in magnitude; a NaN, an infinity or a larger entry makes the output block NaN.  Waits are
-// bounded (pm_umma.cuh).
+// bounded (pm_umma.cuh): once one gave up, the products leave their output as it was, and the callers turn the leaf or the
+// gradient into NaN beside the status bit.
 #pragma once
 
 #include "pm_fxl.cuh"

@@ -422,9 +422,13 @@ __device__ __forceinline__ void adjoint_large_body(const GradParams &p, void *sc
                     const int sl = p.slot_of[raw];
                     return sl >= 0 ? Ttr[sl] : Cx<Real>::make(Real(0), Real(0));
                 };
+                Real gs = gscale;
+                if constexpr (kUmma) {  // a wait gave up: products were skipped
+                    if (*(volatile int *)uc->abort) gs = (Real)nan("");
+                }
                 auto emit = [&](int k, int64_t sidx, C qv) {
                     Real *gr = (Real *)p.grad + (size_t)k * p.S + sidx;
-                    const Real v = gscale * (zr * qv.y - zi * qv.x);
+                    const Real v = gs * (zr * qv.y - zi * qv.x);
                     if (INTEG == kSimpson) atomicAdd(gr, v);  // end points are shared by two slices
                     else *gr = v;
                 };

@@ -595,7 +595,8 @@ __device__ __forceinline__ void large_body(const FusedParams &p, typename Cx<Rea
 // x = q 2^-56 (every one is bounded, see pm_digits.cuh), so that the operands of the tcgen05 products are split without a
 // conversion and the Horner passes leave the FP64 pipe.  Sixteen warps: the splits and sums are chains of integer
 // instructions, and eight warps of 255 registers issued one instruction per cycle of the SM's four.  A norm without a class
-// (NaN, infinite) makes the leaf NaN.
+// (NaN, infinite) makes the leaf NaN, and so does a wait that gave up: the products after it are skipped and leave what was in
+// their buffers.
 constexpr int kUmmaThreads = 512;
 template <int D, int INTEG>
 __device__ __forceinline__ void large_body_fx(const FusedParams &p, longlong2 *ws, int blk, int nblk, unsigned char *smem,
@@ -613,6 +614,7 @@ __device__ __forceinline__ void large_body_fx(const FusedParams &p, longlong2 *w
     const int64_t j0 = p.n_steps * blk / nblk;
     const int len = (int)(p.n_steps * (blk + 1) / nblk - j0);
     const bool traj = p.traj_out != nullptr;
+    auto gave_up = [&]() { return *(volatile int *)uc.abort != 0; };  // uniform: every product ends with a barrier
     if (tid == 0) s_bad = 0;
     __syncthreads();
     for (int i = ti; i < ext; i += NT / 16)
@@ -641,7 +643,7 @@ __device__ __forceinline__ void large_body_fx(const FusedParams &p, longlong2 *w
         }
         __syncthreads();
         const int code = s_code;
-        const double bad = s_bad ? nan("") : 0.0;
+        const bool slice_bad = s_bad != 0;  // read here: thread 0 sets it for the next slice while others still write outputs
         const int q = cls_q(code), rh = cls_r(code), s = cls_s(code) + p.extra_squarings;
         double *gpk = D <= 128 ? (double *)smem : (double *)P0;
         // packed exponent sum_b gamma_b P_b, two columns per thread
@@ -723,6 +725,7 @@ __device__ __forceinline__ void large_body_fx(const FusedParams &p, longlong2 *w
         if (traj && ((j + 1) % p.traj_every == 0 || j + 1 == p.n_steps)) {
             const int64_t o = j / p.traj_every;
             const int d = p.d_out;
+            const double bad = slice_bad || gave_up() ? nan("") : 0.0;
             if (p.traj_psi0 == nullptr) {
                 for (int e = tid; e < d * d; e += NT) {
                     const longlong2 v = SR[(e / d) * D + e % d];
@@ -764,7 +767,7 @@ __device__ __forceinline__ void large_body_fx(const FusedParams &p, longlong2 *w
     }
     if (flags) atomicOr(&p.status[0], flags);
     // block partial (the leaf product) as doubles, the identity beyond the dimension
-    const double bad = s_bad ? nan("") : 0.0;
+    const double bad = s_bad || gave_up() ? nan("") : 0.0;
     for (int e = tid; e < DD; e += NT) {
         double2 v = make_double2((e / D) == (e % D) ? 1.0 : 0.0, 0.0);
         if (max(e / D, e % D) < p.d_out) v = make_double2(fx::to_double(SR[e].x) + bad, fx::to_double(SR[e].y) + bad);
