@@ -206,6 +206,17 @@ int ws_reserve(parament_ctx *ctx, Workspace &w, size_t bytes) {
     return PARAMENT_OK;
 }
 
+// digits of the kept basis matrices for the traces of the gradient (D = 8, 16)
+int fx_trace_build(parament_ctx *ctx, int Dp) {
+    const int nb = ctx->nb_eff;
+    const int st = ws_reserve(ctx, ctx->fxtrace, Dp == 8 ? fx_trace_bytes_d8(nb) : fx_trace_bytes_d16(nb));
+    if (st) return st;
+    PM_CUDA((Dp == 8 ? fx_trace_d8 : fx_trace_d16)((const double *)ctx->cpacked64.ptr, (const double *)ctx->cbnorm.ptr, nb,
+                                                  ctx->fxtrace.ptr, ctx->stream));
+    ctx->fxtrace_ready = true;
+    return PARAMENT_OK;
+}
+
 void ws_free(Workspace &w) {
     if (w.ptr) cudaFree(w.ptr);
     w.ptr = nullptr;
@@ -963,7 +974,10 @@ int parament_set_hamiltonians(parament_ctx *ctx, int dim, int n_ctrl, const void
                                                       kept, ctx->fxbasis.ptr, ctx->stream));
     }
     ctx->nb_eff = kept;
+    // the trace digits: by the first gradient of the context, from then on here, with the other forms of the basis, so that a
+    // captured gradient neither holds their kernel nor replays with those of other Hamiltonians
     ctx->fxtrace_ready = false;
+    if (ctx->fxtrace.ptr && (Dp == 8 || Dp == 16) && (st = fx_trace_build(ctx, Dp))) return st;
 
     ctx->dim = dim;
     ctx->dpad = Dp;
@@ -1387,13 +1401,7 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
         asmem = ctx->smem_optin;
         if ((st = ws_reserve(ctx, ctx->fxadj, (size_t)L * (Dp == 8 ? fx_adjoint_leaf_bytes_d8() : fx_adjoint_leaf_bytes_d16()))))
             return st;
-        if (!ctx->fxtrace_ready) {
-            const int nb = ctx->nb_eff;
-            if ((st = ws_reserve(ctx, ctx->fxtrace, Dp == 8 ? fx_trace_bytes_d8(nb) : fx_trace_bytes_d16(nb)))) return st;
-            PM_CUDA((Dp == 8 ? fx_trace_d8 : fx_trace_d16)((const double *)ctx->cpacked64.ptr,
-                                                          (const double *)ctx->cbnorm.ptr, nb, ctx->fxtrace.ptr, ctx->stream));
-            ctx->fxtrace_ready = true;
-        }
+        if (!ctx->fxtrace_ready && (st = fx_trace_build(ctx, Dp))) return st;
     } else if (large) {
         asmem = adjoint_large_smem(Dp, fp64);
         if (asmem > ctx->smem_optin)
