@@ -131,7 +131,8 @@ typedef enum {
        workspace cap); leaves longer than a sub-chunk are re-computed from checkpoints.  FP64 with d >= 5 keeps
        no prefixes: reported, without effect */
     PARAMENT_OPT_GRAD_SUBCHUNK = 8,
-    /* gradient: cap in MiB on the per-slice prefix buffer of the adjoint sweep (default 4096) */
+    /* gradient: cap in MiB on the per-slice prefix buffer of the adjoint sweep (default 4096); FP64 with d in 5..16 and what
+       runs on it: on the sweep's workspace per leaf (24 KiB for d <= 8, 120 KiB above; at least one leaf's) */
     PARAMENT_OPT_WORKSPACE_MB = 9,
     /* batched: target slices per leaf (0 = by dimension: 8 for d > 16, 16 for d in 9..16, else 64) */
     PARAMENT_OPT_BATCH_LEAF_STEPS = 10,

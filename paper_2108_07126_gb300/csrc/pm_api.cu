@@ -1395,12 +1395,15 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     // adjoint launch geometry: d <= 16 warp groups over a persistent grid, d > 16 one block per leaf
     int aw = 8, agrid = 0;
     size_t asmem = 0;
-    int64_t TG = 0;
+    int64_t TG = 0, fx_slots = 0;
+    const size_t cap = (size_t)ctx->opt_workspace_mb << 20;
     const bool fx_adjoint = fp64 && (Dp == 8 || Dp == 16);  // one warp per leaf on the digit products, one sweep
     if (fx_adjoint) {
+        const size_t leaf_bytes = Dp == 8 ? fx_adjoint_leaf_bytes_d8() : fx_adjoint_leaf_bytes_d16();
         asmem = ctx->smem_optin;
-        if ((st = ws_reserve(ctx, ctx->fxadj, (size_t)L * (Dp == 8 ? fx_adjoint_leaf_bytes_d8() : fx_adjoint_leaf_bytes_d16()))))
-            return st;
+        agrid = ctx->sm_count;
+        fx_slots = std::min<int64_t>(L, std::max<int64_t>(1, (int64_t)(cap / leaf_bytes)));
+        if ((st = ws_reserve(ctx, ctx->fxadj, (size_t)fx_slots * leaf_bytes))) return st;
         if (!ctx->fxtrace_ready && (st = fx_trace_build(ctx, Dp))) return st;
     } else if (large) {
         asmem = adjoint_large_smem(Dp, fp64);
@@ -1420,7 +1423,6 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     const int64_t maxlen = L > 0 ? (N + L - 1) / L : 0;
     int64_t c_sub = ctx->opt_grad_subchunk > 0 ? ctx->opt_grad_subchunk : std::max<int64_t>(maxlen, 1);
     const size_t csz = 2 * rsz;  // complex element
-    const size_t cap = (size_t)ctx->opt_workspace_mb << 20;
     while (c_sub > 1 && (size_t)TG * c_sub * DD * csz > cap) c_sub = (c_sub + 1) / 2;
     const int64_t n_ckpt = std::max<int64_t>(1, (maxlen + c_sub - 1) / c_sub);
     if (!fx_adjoint && !(large && fp64)) {  // one sweep stores no prefixes
@@ -1479,6 +1481,7 @@ int parament_propagate_grad(parament_ctx *ctx, const void *V, double *loss_out, 
     gp.fx_basis = ctx->fxbasis.ptr;
     gp.fx_trace = ctx->fxtrace.ptr;
     gp.fx_g = ctx->fxadj.ptr;
+    gp.fx_slots = fx_slots;
     {
         const double u = fp64 ? std::ldexp(1.0, -53) : std::ldexp(1.0, -24);
         FusedParams tmp;

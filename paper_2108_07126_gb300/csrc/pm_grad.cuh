@@ -58,7 +58,8 @@ struct GradParams {
     double coef_d[kMaxDegree + 1];
     float coef_f[kMaxDegree + 1];
     const void *fx_basis, *fx_trace;  // digit path (pm_fx_grad.cuh): digits of the basis for the exponents and the traces
-    void *fx_g;                       // digit path: workspace per leaf
+    void *fx_g;                       // digit path: workspace of fx_slots warps
+    int64_t fx_slots, fx_leaf0;       // leaves of a launch and its first one
 };
 
 struct ScanParams {

@@ -21,19 +21,19 @@ static int adjoint_occupancy(int warps, size_t smem) {
     return e == cudaSuccess ? nb : 0;
 }
 
-// scans, then the adjoint: FP32 by groups of lanes on the CUDA cores, FP64 by the digit products (smem: the shared
-// memory limit of a block there)
+// scans, then the adjoint: FP32 by groups of lanes on the CUDA cores, FP64 by the digit products (grid: the
+// number of SMs, smem: the shared memory limit of a block there)
 cudaError_t grad_run_d16(int fp64, int integ, const ScanParams &sp, const GradParams &gp, int grid, int warps,
                          size_t smem, cudaStream_t st) {
     cudaError_t e = fx::scan_run<16>(sp, sp.bpin, true, st);
     if (e != cudaSuccess) return e;
     switch (integ * 2 + (fp64 ? 1 : 0)) {
         case 0: return adjoint_launch<float, kMidpoint>(gp, grid, warps, smem, st);
-        case 1: return fx::adjoint_launch<16, kMidpoint>(gp, smem, st);
+        case 1: return fx::adjoint_launch<16, kMidpoint>(gp, grid, smem, st);
         case 2: return adjoint_launch<float, kGL2>(gp, grid, warps, smem, st);
-        case 3: return fx::adjoint_launch<16, kGL2>(gp, smem, st);
+        case 3: return fx::adjoint_launch<16, kGL2>(gp, grid, smem, st);
         case 4: return adjoint_launch<float, kSimpson>(gp, grid, warps, smem, st);
-        case 5: return fx::adjoint_launch<16, kSimpson>(gp, smem, st);
+        case 5: return fx::adjoint_launch<16, kSimpson>(gp, grid, smem, st);
     }
     return cudaErrorInvalidValue;
 }
