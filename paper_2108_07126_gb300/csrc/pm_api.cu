@@ -1066,7 +1066,7 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
     if (Dp > kMaxSmallDim) {
         // one thread block per leaf (512 threads for FP64 slices of d > 32 on tcgen05, else 256); working matrices in a
         // per-block scratch region
-        warps = fp64 && Dp >= 64 && !ctx->opt_exp_method ? 16 : 8;
+        warps = fp64 && Dp >= 64 && !cheb ? 16 : 8;
         smem = large_smem(Dp, fp64, nb, tc);
         if (smem > ctx->smem_optin) return set_err(ctx, PARAMENT_ERR_UNSUPPORTED, "large-d shared memory %zu B", smem);
         int bps = large_blocks_per_sm(Dp, fp64, (int)ctx->integ, smem, tc);
