@@ -77,3 +77,31 @@ def test_forced_degree_and_extra_squarings(prop, d, prec, degree, extra):
         assert squarings >= extra and st["exp_products"] >= n * extra
     else:
         assert st["exp_products"] == 0 and st["max_degree"] == (15 if prec == "fp64" else 11)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("w", [0.6875, -3.0, 77.0])
+@pytest.mark.parametrize("n,grid,warps", [(100, 0, 0), (16384, 0, 0), (16384, 1, 1), (300001, 0, 0)])
+def test_phases_add_up_exactly(prop, n, grid, warps, w, prec):
+    """H = (w + c_j) I with exponents that are exact in the precision, but not their sums: U = e^{-i sum} I.  The phases are summed
+    as integers, so what is left is the reduction of a slice's phase above 4 rad (2^-60 a slice), the angle's (2^-52) and the
+    cosine's and sine's rounding, and with complex64 that of U."""
+    from fractions import Fraction
+
+    import torch
+
+    from paper_2108_07126_gb300 import binding as b
+
+    bits = 46 if prec == "fp64" else 8  # c: multiples of 2^-bits up to 1 / 4
+    k = np.random.default_rng(n).integers(-(1 << (bits - 2)), (1 << (bits - 2)) + 1, (1, n))
+    hd, cd = (torch.complex128, torch.float64) if prec == "fp64" else (torch.complex64, torch.float32)
+    prop.set_option(b.PARAMENT_OPT_GRID_BLOCKS, grid)
+    prop.set_option(b.PARAMENT_OPT_BLOCK_WARPS, warps)
+    prop.set_hamiltonians(torch.eye(2, dtype=hd) * w, torch.eye(2, dtype=hd)[None], "midpoint")
+    prop.set_controls(torch.as_tensor(k * 2.0 ** -bits).to(cd), 0.25, n)
+    U = prop.propagate(prec).cpu().numpy()
+    phi = (n * Fraction(w) + Fraction(int(k.sum()), 1 << bits)) / 4
+    two_pi = 2 * Fraction("3.14159265358979323846264338327950288419716939937510")
+    phi = float(phi - round(phi / two_pi) * two_pi)
+    tol = n * 2.0 ** -60 + 2.0 ** -50 + (0 if prec == "fp64" else 2.0 ** -23)
+    assert np.max(np.abs(U - np.exp(-1j * phi) * np.eye(2))) <= tol
