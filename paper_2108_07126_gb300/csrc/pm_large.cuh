@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(large_tcm<Real, D, TC>() == 6 ? kUmmaThreads :
     } else {
         large_body<Real, D, INTEG, TCM>(p, ws, blockIdx.x, gridDim.x, smem);
     }
-    // the pairwise tree over the block partials runs in tree_level_kernel launches
+    // the pairwise tree over the block partials runs in launches of its own (launch_large)
 }
 
 // FP64, D >= 64 with the Chebyshev exponential, whose recurrence leaves the fixed-point range: products on the FP64 pipe
@@ -836,8 +836,8 @@ __global__ void __launch_bounds__(kLargeThreads, 1) large_cheb_kernel(const Fuse
 // block's scratch), the first one leaves; the root writes U_out and snapshots
 // the statistics.  As in the single-problem tree, the levels with at most 8
 // nodes multiply in FP64 and the levels below in Real (the partials stay FP64
-// in global memory): an FP64 product of two 64 x 64 matrices costs an SM
-// ~0.5 M cycles on GB300's FP64 pipe, as much as the FP32 work of ~5 slices.
+// in global memory).  FP64: digit products, but at D = 128 in the FP32 kernels,
+// where their panels would cost the second block per SM (the FP64 pipe then).
 template <typename Real, int D>
 __device__ void large_arrival_tree(const FusedParams &p, void *ws_bytes, int blk, int nblk, unsigned char *smem) {
     constexpr int DD = D * D;
@@ -898,14 +898,13 @@ __device__ void large_arrival_tree(const FusedParams &p, void *ws_bytes, int blk
 
 // One level of the pairwise tree over block partials (Sec. 2.2) for large D:
 // out[i] = in[2i+1] * in[2i] (the later partial on the left), an odd last
-// partial is carried.  Storage is FP64; the products are computed in Real
-// (FP64 for the top levels, FP32 below them in the FP32 modes).  Each block
-// computes one 32 x 32 tile of one product, so a level spreads over the GPU.
-// The last level (one output) also writes U_out and snapshots the statistics.
-template <typename Real, int D>
+// partial is carried.  The lower levels of the FP32 modes: partials in FP64,
+// products in FP32 (the top levels, and all of FP64: tree_level_fx_kernel).
+// Each block computes one 32 x 32 tile of one product, so a level spreads over the GPU.
+template <int D>
 __global__ void __launch_bounds__(256) tree_level_kernel(const double2 *__restrict__ in, int n_in,
-                                                         double2 *__restrict__ out, const FusedParams p) {
-    using C = typename Cx<Real>::T;
+                                                         double2 *__restrict__ out) {
+    using C = float2;
     constexpr int T = 32, KP = 16;
     __shared__ C As[T][KP + 1], Bs[KP][T + 1];
     const int tiles = D / T;
@@ -920,16 +919,16 @@ __global__ void __launch_bounds__(256) tree_level_kernel(const double2 *__restri
 #pragma unroll
     for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int c = 0; c < 2; ++c) acc[r][c] = Cx<Real>::make(0, 0);
+        for (int c = 0; c < 2; ++c) acc[r][c] = make_float2(0.f, 0.f);
     if (has_pair) {
         for (int k0 = 0; k0 < D; k0 += KP) {
             for (int e = threadIdx.x; e < T * KP; e += blockDim.x) {
                 const int r = e / KP, k = e % KP;
                 const double2 a = R[(size_t)(ti * T + r) * D + k0 + k];
-                As[r][k] = Cx<Real>::make((Real)a.x, (Real)a.y);
+                As[r][k] = make_float2((float)a.x, (float)a.y);
                 const int kb = e / T, cb = e % T;
                 const double2 b = L[(size_t)(k0 + kb) * D + tj * T + cb];
-                Bs[kb][cb] = Cx<Real>::make((Real)b.x, (Real)b.y);
+                Bs[kb][cb] = make_float2((float)b.x, (float)b.y);
             }
             __syncthreads();
 #pragma unroll
@@ -952,18 +951,7 @@ __global__ void __launch_bounds__(256) tree_level_kernel(const double2 *__restri
             const double2 v = has_pair ? make_double2((double)acc[r][c].x, (double)acc[r][c].y)
                                        : L[(size_t)i * D + j];
             O[(size_t)i * D + j] = v;
-            if (gridDim.y == 1 && n_in <= 2) {  // last level: the propagator itself
-                const int d = p.d_out;
-                if (i < d && j < d) {
-                    if (p.out_c128) ((double2 *)p.U_out)[i * d + j] = v;
-                    else ((float2 *)p.U_out)[i * d + j] = make_float2((float)v.x, (float)v.y);
-                }
-            }
         }
-    if (gridDim.y == 1 && n_in <= 2 && blockIdx.x == 0 && threadIdx.x == 0) {
-        for (int i = 0; i < 4; ++i) p.counters[4 + i] = atomicExch(&p.counters[i], 0ull);
-        p.status[1] = atomicExch(&p.status[0], 0u);
-    }
 }
 
 template <int T, int D> __device__ __forceinline__ void zero_tile(double2 *O) {
@@ -971,7 +959,8 @@ template <int T, int D> __device__ __forceinline__ void zero_tile(double2 *O) {
     __syncthreads();
 }
 
-// The same level with FP64 products on the digit products: block (tile, pair) computes one 32 x 32 tile.
+// The same level with FP64 products on the digit products: block (tile, pair) computes one 32 x 32 tile.  The last level (one
+// output) also writes U_out and snapshots the statistics.
 // D = 128, one product: 16 blocks of 14 k cycles against 16 blocks of 308 k on the FP64 pipe.
 template <int D>
 __global__ void __launch_bounds__(256) tree_level_fx_kernel(const double2 *__restrict__ in, int n_in,
@@ -1089,7 +1078,7 @@ cudaError_t launch_large(const FusedParams &p, void *scratch, int grid, size_t s
         if (std::is_same<Real, double>::value || n <= 8)
             tree_level_fx_kernel<D><<<g, 256, fxl::G<32>::BYTES, st>>>(bufs[cur], n, bufs[cur ^ 1], p);
         else
-            tree_level_kernel<float, D><<<g, 256, 0, st>>>(bufs[cur], n, bufs[cur ^ 1], p);
+            tree_level_kernel<D><<<g, 256, 0, st>>>(bufs[cur], n, bufs[cur ^ 1]);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         cur ^= 1;
         n = n_out;
