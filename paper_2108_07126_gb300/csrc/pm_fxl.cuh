@@ -47,10 +47,12 @@ __device__ __forceinline__ i64 to_fixed(double v, bool &bad) {
     return (i64)b < 0 ? -(i64)q : (i64)q;
 }
 
+// COMPACT: fewer registers (one part of A at a time, the parts in a loop).  For the batched FP32 kernel: with the full form in its
+// tree, ptxas spilled in the items of small d (64 instances, d = 4, N = 10 000: 385 -> 568 us, with this one 410 us).
 // C = A B for one block of at most BM x BM: A is rows x K (row stride lda), B is K x cols (ldb), C (ldc) must not
 // alias them; rows, cols and K are multiples of 16 (BM = 32: rows and cols full).  All 256 threads; smem:
 // G<BM>::BYTES.  Starts after the caller's barrier and ends with one.
-template <int BM>
+template <int BM, bool COMPACT = false>
 __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double2 *B, int ldb, double2 *C, int ldc, int K,
                                          unsigned char *smem, int rows = BM, int cols = BM) {
     using g = G<BM>;
@@ -120,12 +122,14 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
         if (more) load((kp + 1) * KP);
         const uint32_t *sa = st + (kp & 1) * (g::AW + g::BW), *sb = sa + g::AW;
         fx::Digits<16> a;
+        if constexpr (!COMPACT) {
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
             const uint4 x = *reinterpret_cast<const uint4 *>(sa + rb * (2 * ND * 128) + 2 * i * 128 + lane * 4);
             const uint4 y = *reinterpret_cast<const uint4 *>(sa + rb * (2 * ND * 128) + (2 * i + 1) * 128 + lane * 4);
             a.re[i][0] = x.x; a.re[i][1] = x.y; a.re[i][2] = x.z; a.re[i][3] = x.w;
             a.im[i][0] = y.x; a.im[i][1] = y.y; a.im[i][2] = y.z; a.im[i][3] = y.w;
+        }
         }
 #pragma unroll
         for (int t = 0; t < NTW; ++t) {
@@ -136,6 +140,34 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
             }
             if (t >= ntw || rb >= nrb) continue;
             const uint32_t *sn = sb + (cw * ntw + t) * (2 * ND * 64) + lane * 2;
+            if constexpr (COMPACT) {
+#pragma unroll 2
+                for (int pt = 0; pt < 2; ++pt) {
+                    float acc[fx::NA][4];
+                    fx::acc_init(acc);
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {  // Ar, then Ai
+                        uint4 x[ND];
+                        uint2 b[ND];
+                        const uint32_t neg = h == 1 && pt == 0 ? 0x80008000u : 0u;
+#pragma unroll
+                        for (int i = 0; i < ND; ++i) x[i] = *reinterpret_cast<const uint4 *>(sa + rb * (2 * ND * 128) + (2 * i + h) * 128 + lane * 4);
+#pragma unroll
+                        for (int j = 0; j < ND; ++j) {
+                            b[j] = *reinterpret_cast<const uint2 *>(sn + (2 * j + (h ^ pt)) * 64);
+                            b[j].x ^= neg;
+                            b[j].y ^= neg;
+                        }
+#pragma unroll
+                        for (int i = 0; i < ND; ++i)
+#pragma unroll
+                            for (int j = 0; j <= fx::last_digit(i); ++j) fx::mma(acc[i + j], x[i].x, x[i].y, x[i].z, x[i].w, b[j].x, b[j].y);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) o[t][pt][u] += fx::collect_fine(acc, u);
+                }
+                continue;
+            }
 #pragma unroll
             for (int pt = 0; pt < 2; ++pt) {  // Re: Ar Br + Ai (-Bi); Im: Ar Bi + Ai Br
                 float acc[fx::NA][4];
@@ -186,14 +218,14 @@ __device__ __forceinline__ void block_mm(const double2 *A, int lda, const double
 // or B; ends with a barrier.  Only the leading ceil(d / 16) * 16 rows, columns and k are read and written: d = 40 in
 // its 64 x 64 frame takes 3 of 4 panels on 3 of 4 row blocks.
 __device__ __forceinline__ int extent(int d) { return (d + 15) & ~15; }
-template <int D> __device__ __noinline__ void cta_mm(const double2 *A, const double2 *B, double2 *C, unsigned char *smem, int d) {
-    constexpr int BM = block_of<D>();
+template <int D, int BM = block_of<D>(), bool COMPACT = false>
+__device__ __noinline__ void cta_mm(const double2 *A, const double2 *B, double2 *C, unsigned char *smem, int d) {
     const int n = D == 32 ? 32 : extent(d);
 #pragma unroll 1
     for (int i = 0; i < n; i += BM)
 #pragma unroll 1
         for (int j = 0; j < n; j += BM)
-            block_mm<BM>(A + (size_t)i * D, D, B + j, D, C + (size_t)i * D + j, D, n, smem, min(BM, n - i), min(BM, n - j));
+            block_mm<BM, COMPACT>(A + (size_t)i * D, D, B + j, D, C + (size_t)i * D + j, D, n, smem, min(BM, n - i), min(BM, n - j));
 }
 
 }  // namespace fxl

@@ -861,7 +861,8 @@ __device__ void large_arrival_tree(const FusedParams &p, void *ws_bytes, int blk
                     R2[e] = __ldcg(gR + e);
                 }
                 __syncthreads();
-                if constexpr (std::is_same<Real, double>::value || tree_on_digits<D>()) fxl::cta_mm<D>(R2, L2, gL, smem, p.d_out);
+                if constexpr (std::is_same<Real, double>::value) fxl::cta_mm<D>(R2, L2, gL, smem, p.d_out);
+                else if constexpr (tree_on_digits<D>()) fxl::cta_mm<D, 32, true>(R2, L2, gL, smem, p.d_out);
                 else cta_mm<double, D>(R2, L2, gL, smem);
             } else {
                 float2 *Lf = (float2 *)ws_bytes, *Rf = Lf + DD, *Cf = Rf + DD;
