@@ -1121,8 +1121,15 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
         grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)(fp64 ? 4 : 8) * ctx->sm_count));
     }
     if (grid <= 0) {
-        const int lm = fp64 ? kLeafMinSteps64 : kLeafMinSteps;
-        const int64_t need = (ctx->n_steps + (int64_t)leaves_per_block * lm - 1) / ((int64_t)leaves_per_block * lm);
+        auto blocks_of = [&](int slices) {
+            return (ctx->n_steps + (int64_t)leaves_per_block * slices - 1) / ((int64_t)leaves_per_block * slices);
+        };
+        int64_t need = blocks_of(fp64 ? kLeafMinSteps64 : kLeafMinSteps);
+        // FP32 of d <= 4 (256 leaves a block, one thread each): a block's trees cost several slices, so beyond a sixth of the
+        // SMs leaves grow to eight slices before more blocks are taken.  d = 4, grid 25 / 50 / 100 / 152: N = 25600 80 / 90 / 121 /
+        // 131 us, 51200 99 / 99 / 126 / 170, 102400 137 / 119 / 136 / 174, 204800 215 / 157 / 156 / 189, 409600 374 / 234 / 193 /
+        // 213; states, d = 2, N = 102400 371 / 370 / 427 / 504.
+        if (!fp64 && Dp <= 4) need = std::min(need, std::max<int64_t>(blocks_of(8), ctx->sm_count / 6));
         grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)bps * ctx->sm_count));
     }
     grid = std::min(grid, ctx->max_grid);

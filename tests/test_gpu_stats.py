@@ -28,3 +28,31 @@ def test_gradient_threads_with_the_chebyshev_option(d):
         assert threads[0] == threads[1] and torch.equal(grads[0], grads[1])
     finally:
         prop.close()
+
+
+@pytest.mark.parametrize("d", [3, 4])
+@pytest.mark.parametrize("n", [1, 511, 513, 12800, 12801, 51201, 102400, 330000])
+def test_fp32_leaves_of_small_systems(d, n):
+    """d = 3, 4, FP32: two slices a leaf up to a sixth of the SMs, then up to eight, then more blocks; U(T) against FP64."""
+    import torch
+
+    from paper_2108_07126_gb300 import binding as b
+    from tolerances import tol32
+
+    prob = wl.random_problem(d, 2, n, "midpoint", seed=7000 + d, g_norm=0.3)
+    H0, Hk, c = prob.H0.astype(np.complex64), prob.Hk.astype(np.complex64), prob.c.astype(np.float32)
+    prop = b.Propagator(0)
+    try:
+        U = {}
+        for prec, hd, cd in (("fp32", torch.complex64, torch.float32), ("fp64", torch.complex128, torch.float64)):
+            prop.set_hamiltonians(torch.as_tensor(H0).to(hd), torch.as_tensor(Hk).to(hd), "midpoint")
+            prop.set_controls(torch.as_tensor(c).to(cd), prob.dt, n)
+            U[prec] = prop.propagate(prec).cpu().numpy()
+            if prec == "fp32":
+                st = prop.stats()
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        leaf = n / st["leaves"]
+        assert st["grid_blocks"] <= max(sms // 6, -(-n // (8 * 256))) and (leaf <= 8 or st["grid_blocks"] >= sms)
+        assert np.max(np.abs(U["fp32"] - U["fp64"])) <= tol32(d, n)
+    finally:
+        prop.close()
