@@ -80,12 +80,16 @@ typedef enum {
 /*
  * Arithmetic of the exponential and of the product tree.
  *  FP64: double inputs, results and coefficients.  d >= 5: the complex products and the exponents run in 64-bit fixed
- *        point with exact sums (tensor cores, base-256 digits; absolute rounding 2^-57 on matrices of norm about one,
- *        the size of a double's rounding there); d <= 4, the Chebyshev option, batched items of d <= 16 and
- *        parament_propagate_noalloc: double arithmetic throughout.
+ *        point with exact sums (tensor cores, base-256 digits).  The matrices have norms about one and every operation rounds
+ *        an entry by at most 2^-57 in absolute terms: in norm that is no more than double arithmetic, but entries far below one
+ *        keep fewer relative digits than a double has (weak couplings, very short steps: with slice exponents of 6e-8 and U a
+ *        rotation by 3e-8, the small entries are off by about 1e-15, in double arithmetic by less than 1e-20).
+ *        Double arithmetic: d <= 4; the slices and the products within a thread block of the Chebyshev option, of batched
+ *        items of d <= 16 and of parament_propagate_noalloc (their products between blocks are fixed point from d = 5 on).
  *  FP32: exponent assembly, exponential and the in-block tree in float; the
  *        norm bound that picks the Taylor degree and the number of squarings,
- *        and the product tree above the thread-block level, in double.
+ *        and the product tree above the thread-block level, in double
+ *        (d >= 5: the 64-bit fixed point of FP64).
  *  FP32_TC_TF32X3: FP32 with the complex products of large d on the tensor
  *        cores: every FP32 operand split into two round-to-nearest TF32 terms,
  *        three MMAs per real product (hi*hi + hi*lo + lo*hi), FP32 accumulation
@@ -118,8 +122,9 @@ typedef enum {
     PARAMENT_OPT_TAYLOR_DEGREE = 1,
     /* thread blocks of the fused kernel; 0 (default) = fill every SM */
     PARAMENT_OPT_GRID_BLOCKS = 2,
-    /* warps per thread block; 0 (default) = largest that fits shared memory (at most 16 for FP32
-       d in 9..16, 16 for FP64 d in 5..8, 8 otherwise; d <= 2: 4, or what a single block needs) */
+    /* warps per thread block; 0 (default) = largest that fits shared memory (at most 12 for FP32
+       d in 9..16, 16 for FP64 d in 5..8, 8 otherwise; FP64 takes fewer where that spreads a short run; U(T) of d <= 2: 4, or
+       what a single block needs) */
     PARAMENT_OPT_BLOCK_WARPS = 3,
     /* 1 (default) = reject non-Hermitian H in set_hamiltonians; 0 = skip the check */
     PARAMENT_OPT_CHECK_HERMITIAN = 4,
@@ -147,7 +152,7 @@ typedef enum {
        (PARAMENT_ERR_UNSUPPORTED); the gradient always uses the Taylor exponential */
     PARAMENT_OPT_EXP_METHOD = 13,
     /* FP32 and tensor-core precisions: 1 (default) = one Newton-Schulz step R <- R (3 I - R^dagger R) / 2
-       on every leaf product (the exact product is unitary; FP32 rounding that repeats from slice to
+       on every leaf product, or with d <= 16 and leaves of at most 16 slices on the block's product (the exact product is unitary; FP32 rounding that repeats from slice to
        slice, and the truncating tensor-core accumulation, otherwise drift R off the unitary group
        linearly in the leaf length); 0 = plain products */
     PARAMENT_OPT_UNITARY_STEP = 14,
@@ -178,13 +183,14 @@ typedef struct {
 /* product back-ends reported in parament_stats.product_backends (a batched call ORs the
    back-ends of its dimension classes) */
 #define PARAMENT_BACKEND_CUDA_CORES 0x1u /* the precision's own arithmetic: FP32 / FP64 fused multiply-adds, or the
-                                            exact integer-digit products of FP64 */
+                                            exact integer-digit products of FP64 (on mma.sync, d >= 33 on tcgen05) */
 #define PARAMENT_BACKEND_MMA_SYNC 0x2u   /* reduced-precision products by warp-level mma.sync (no path of this build) */
 #define PARAMENT_BACKEND_TCGEN05 0x4u    /* tcgen05.mma with tensor-memory accumulators */
 
 #define PARAMENT_DEV_NONFINITE_NORM 0x1u /* a slice's norm bound was NaN/Inf */
 #define PARAMENT_DEV_NORM_CAPPED 0x2u    /* a norm exceeded the largest scaling in the table */
-#define PARAMENT_DEV_TENSOR_TIMEOUT 0x4u /* a bounded tensor-core wait gave up; the result is invalid */
+#define PARAMENT_DEV_TENSOR_TIMEOUT 0x4u /* a bounded tensor-core wait gave up (3xTF32, BF16x3, FP64 of d >= 33); the result is
+                                            invalid (FP64: NaN) */
 
 /* Library version as major * 1000 + minor. */
 int parament_version(void);
@@ -259,10 +265,10 @@ int parament_propagate(parament_ctx *ctx, void *U_out, parament_precision prec);
  * dX_j/dc = -i sum_e (d gamma_e / dc) B_e over the effective-control basis (Sec. 4, Eq.
  * magnus_coeffs: H0, H_k, i[H0, H_k], i[H_k, H_l]), and L_X the Frechet derivative of exp, taken
  * as the upper-right block of exp([[X, Lambda], [0, X]]).  The prefixes P and suffixes S come from
- * the forward tree: leaf and block products of the forward kernel, exclusive scans over them, then
- * per leaf a forward sweep (prefixes, re-computed from checkpoints for long leaves) and a backward
- * sweep; FP64 of d >= 5 undoes the slices in one backward sweep instead, and FP32 of d = 5..8 up to 2048
- * slices is computed in FP64 and rounded.  A Simpson end sample belongs to two slices and receives both contributions.  d <= 16:
+ * the forward tree: leaf and block products of the forward kernel and exclusive scans over them.  Per leaf,
+ * FP32 and FP64 of d <= 4 run a forward sweep (prefixes, re-computed from checkpoints for long leaves) and a
+ * backward one; FP64 of d >= 5 keeps no prefixes and undoes the slices in one backward sweep.  FP32 of d = 5..8
+ * up to 2048 slices is computed in FP64 and rounded.  A Simpson end sample belongs to two slices and receives both contributions.  d <= 16:
  * groups of lanes of one warp per leaf; d = 17..256: one thread block per leaf (FP64 Hillis-Steele
  * scans of the leaf products for the prefixes, the suffixes, U(T) and z; block-wide products).
  * V: d x d in the dtype of set_hamiltonians; U_out: optional U(T).  Pointers host or device.

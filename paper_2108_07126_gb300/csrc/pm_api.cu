@@ -85,7 +85,7 @@ constexpr int kMaxDim = 256;
 constexpr int kMaxBatchDim = 128;  // the batched kernel's block-level bodies go up to D = 128
 constexpr int kMaxSmallDim = 16;  // larger dimensions use one thread block per leaf
 // Fewer blocks for short runs: each leaf gets at least two slices.  A slice is a chain of dependent products, dearer than
-// a level of the tree (FP32, 8 -> 2 slices: d = 16, N = 2048 158 -> 94 us, gradient d = 8, N = 1501 600 -> 261 us).
+// a level of the tree (FP32, 8 -> 2 slices: d = 16, N = 2048 158 -> 94 us).
 constexpr int kLeafMinSteps = 2;  // FP32
 // FP32 gradients of d = 5..8 up to this length run in FP64 and round the result: a short run is bound by latency, and the
 // one-sweep FP64 adjoint has less of it (d = 8, FP32 / FP64 path: N = 64 200 / 175 us, 1024 256 / 203 us, 1501 249 / 207 us,
@@ -1094,9 +1094,9 @@ int forward_setup(parament_ctx *ctx, int fp64, void *U_dst, FusedParams &p, int 
         warps = max_warps;
         while (warps > 1 && fused_smem(Dp, fp64, nb, warps, cheb) > ctx->smem_optin) --warps;
         if (fp64 && ctx->opt_grid <= 0) {
-            // an FP64 slice costs ~64x an FP32 one (GB300's FP64 rate), so a short run is spread
+            // an FP64 slice is a long chain, on digits (d >= 5) as on the FP64 pipe, so a short run is spread
             // over more SMs first: halve the warps per block while the grid that gives every leaf
-            // kLeafMinSteps64 slices stays below one block per SM (d = 2, N = 2^14: 8 x 256 ->
+            // kLeafMinSteps64 slices stays below one block per SM (matrix scheme, d = 2, N = 2^14: 8 x 256 ->
             // 128 x 64 threads, 2.2x faster)
             auto blocks_for = [&](int w) {
                 const int64_t per = (int64_t)w * fused_gpw(Dp, fp64, cheb) * kLeafMinSteps64;

@@ -71,7 +71,8 @@ struct FusedParams {
     unsigned long long *counters;
     unsigned *status;
     int extra_squarings;
-    int unitary_step;          // FP32: one Newton-Schulz step R <- R (3 I - R^dagger R) / 2 on every leaf product
+    int unitary_step;          // FP32: one Newton-Schulz step R <- R (3 I - R^dagger R) / 2 on leaf products, or (d <= 16, leaves
+                               // of at most 16 slices) on block products
     int warps;                 // warps of a block that own leaves (0 = all; the others only join the barriers)
     int tc_off;                // batched tensor-core kernel: run this instance's products on the CUDA cores
     const int *cheb_m;         // Chebyshev mode: degree, 1 / beta and coefficients (device, written by
