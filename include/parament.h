@@ -188,7 +188,8 @@ typedef struct {
 #define PARAMENT_BACKEND_TCGEN05 0x4u    /* tcgen05.mma with tensor-memory accumulators */
 
 #define PARAMENT_DEV_NONFINITE_NORM 0x1u /* a slice's norm bound was NaN/Inf */
-#define PARAMENT_DEV_NORM_CAPPED 0x2u    /* a norm exceeded the largest scaling in the table */
+#define PARAMENT_DEV_NORM_CAPPED 0x2u    /* a norm exceeded the largest scaling in the table; the result is not accurate (from d = 5
+                                            on it may be NaN: fixed point holds matrices of norm about one) */
 #define PARAMENT_DEV_TENSOR_TIMEOUT 0x4u /* a bounded tensor-core wait gave up (3xTF32, BF16x3, FP64 of d >= 33); the result is
                                             invalid (FP64: NaN) */
 
