@@ -856,9 +856,19 @@ __device__ void large_arrival_tree(const FusedParams &p, void *ws_bytes, int blk
             double2 *gL = p.partials + (size_t)((idx & ~1) << level) * DD;
             const double2 *gR = p.partials + (size_t)((idx | 1) << level) * DD;
             if (std::is_same<Real, double>::value || n <= 8) {
-                for (int e = tid; e < DD; e += kLargeThreads) {
-                    L2[e] = __ldcg(gL + e);
-                    R2[e] = __ldcg(gR + e);
+                // four elements at a time, all loads before the stores
+                for (int e = tid; e < DD; e += 4 * kLargeThreads) {
+                    double2 l[4], r[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        l[u] = __ldcg(gL + e + u * kLargeThreads);
+                        r[u] = __ldcg(gR + e + u * kLargeThreads);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        L2[e + u * kLargeThreads] = l[u];
+                        R2[e + u * kLargeThreads] = r[u];
+                    }
                 }
                 __syncthreads();
                 if constexpr (std::is_same<Real, double>::value) fxl::cta_mm<D>(R2, L2, gL, smem, p.d_out);
